@@ -274,6 +274,35 @@ __global__ void k_lincomb(T* __restrict__ out, const T* X, double a, const T* Y,
     }
 }
 
+// Em = -Y - B, Ep = Y - B: the factors of a step's tangent map, both with their TF32 split, in
+// one pass over Y and B. Bound by memory: 2 reads and 6 writes of N x ld floats (2 and 2 of
+// doubles); the split products that read the result (hi, lo) leave no use for Em, Ep themselves
+// in FP32, so they are written only where no split is (FP64).
+template <typename T>
+__global__ void k_tangent_factors(T* __restrict__ Em, T* __restrict__ Ep,
+                                  const T* __restrict__ Y, const T* __restrict__ B, size_t nvec,
+                                  T* __restrict__ Em_hi, T* __restrict__ Em_lo,
+                                  T* __restrict__ Ep_hi, T* __restrict__ Ep_lo) {
+    constexpr int W = Vec<T>::W;
+    for (size_t v = blockIdx.x * (size_t)blockDim.x + threadIdx.x; v < nvec;
+         v += (size_t)gridDim.x * blockDim.x) {
+        T y[W], b[W], m[W];
+        load16(Y + v * W, y);
+        load16(B + v * W, b);
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            m[i] = -y[i] - b[i];
+            y[i] = y[i] - b[i];
+        }
+        if (Em) {
+            store16(Em + v * W, m);
+            store16(Ep + v * W, y);
+        }
+        put_split16(Em_hi, Em_lo, v * W, m);
+        put_split16(Ep_hi, Ep_lo, v * W, y);
+    }
+}
+
 // hi/lo split of a contiguous array (float only).
 __global__ void k_split(const float* __restrict__ X, size_t nvec, float* __restrict__ hi,
                         float* __restrict__ lo) {
@@ -672,6 +701,16 @@ cdmpt_status Ew<T>::lincomb(T* out, const T* X, double a, const T* Y, double b, 
                             cudaStream_t s) {
     const size_t nvec = count / Vec<T>::W;
     k_lincomb<T><<<grid_for(nvec), kThreads, 0, s>>>(out, X, a, Y, b, nvec);
+    LAUNCH_CHECK();
+    return CDMPT_OK;
+}
+
+template <typename T>
+cdmpt_status Ew<T>::tangent_factors(T* Em, T* Ep, const T* Y, const T* B, size_t count,
+                                    cudaStream_t s, T* Em_hi, T* Em_lo, T* Ep_hi, T* Ep_lo) {
+    const size_t nvec = count / Vec<T>::W;
+    k_tangent_factors<T><<<grid_for(nvec), kThreads, 0, s>>>(Em, Ep, Y, B, nvec, Em_hi, Em_lo,
+                                                             Ep_hi, Ep_lo);
     LAUNCH_CHECK();
     return CDMPT_OK;
 }

@@ -697,7 +697,7 @@ cdmpt_status launch_oz(int M, int N, int K, const OzOperand& X, const OzOperand&
     p.ey = Y.e;
     const int num_mt = (M + 2 * BM - 1) / (2 * BM);
     const int num_nt = (N + C::BN - 1) / C::BN;
-    p.sym = (ep.sym && M == N && X.s[0] == Y.s[0]) ? 1 : 0;
+    p.sym = (M == N && (ep.sym == 2 || (ep.sym && X.s[0] == Y.s[0]))) ? 1 : 0;
     int tiles = 0;
     if (p.sym)
         for (int j = 0; j < num_nt; ++j) tiles += oz_sym_count(j, num_mt, C::BN);

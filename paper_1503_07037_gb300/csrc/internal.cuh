@@ -181,6 +181,9 @@ struct Ew {
                                  T* hi = nullptr, T* lo = nullptr);
     static cdmpt_status lincomb(T* out, const T* X, double a, const T* Y, double b, size_t count,
                                 cudaStream_t s);
+    // The right and left factors of a step's tangent map: Em = -Y - B, Ep = Y - B, with splits.
+    static cdmpt_status tangent_factors(T* Em, T* Ep, const T* Y, const T* B, size_t count,
+                                        cudaStream_t s, T* Em_hi, T* Em_lo, T* Ep_hi, T* Ep_lo);
     static cdmpt_status transpose(T* out, const T* in, int N, int ld, int blocks, cudaStream_t s,
                                   T* hi = nullptr, T* lo = nullptr);
     static cdmpt_status to_f64(double* out, int ldo, const T* in, int ldi, int N, int rows,
@@ -219,7 +222,8 @@ struct OzEpi {
     const int* ex = nullptr;   // set by gemm_oz from the operands
     const int* ey = nullptr;
     // symmetric result (X is Y, M = N, the C terms symmetric): only the tiles that meet the
-    // upper triangle are computed, each element n >= m written at (m, n) and (n, m)
+    // upper triangle are computed, each element n >= m written at (m, n) and (n, m). 1 holds
+    // only where X is Y; 2 declares the product of two commuting symmetric operands symmetric
     int sym = 0;
 };
 constexpr int kOzDigits = 5;   // digits of the refinement products (39 bits of the row maximum)

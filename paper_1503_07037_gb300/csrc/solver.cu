@@ -16,6 +16,10 @@
 // which makes the CG result about three times more accurate than solving for
 // Z_{k+1} against A_k = I + Z_k^2 directly.
 //
+// First-order maps (response, adjoint): with V_k = A_k^-1 the step Z_{k+1} = 2 Z_k V_k has the
+// tangent dZ_{k+1} = 2 V_k dZ_k V_k - 1/2 Z_{k+1} dZ_k Z_{k+1} (see tangent_step), and
+// V_k = I - 1/2 Z_{k+1} Z_k follows from the stored trajectory without a solve.
+//
 // Chemical potential: Newton on Tr P0 = N_occ with the paper's slope
 // Tr P_mu = beta Tr[P0 (I - P0)] = beta/4 (N - ||Z_n||_F^2) (Eq. NewtRaphs),
 // safeguarded by a bisection bracket. mu1: P1 is linear in mu1 with slope
@@ -1018,7 +1022,7 @@ cdmpt_status Solver<T>::p0_out(Context& cx, double* out, int ldo) {
 
 template <typename T>
 cdmpt_status Solver<T>::gemm_hp(Context& cx, const OzOperand& X, const OzOperand& Y,
-                                const OzEpi& ep) {
+                                const OzEpi& ep, int nd) {
     // a symmetric result computes the tiles of the upper triangle: N (N + 1) N, as for the
     // symmetric TF32 products
     const double flops = ep.sym ? (double)N_ * (N_ + 1) * N_ : 2.0 * N_ * (double)N_ * N_;
@@ -1040,7 +1044,7 @@ cdmpt_status Solver<T>::gemm_hp(Context& cx, const OzOperand& X, const OzOperand
         e1 = cx.ev[2 * cx.ev_used + 1];
         CDMPT_CUDA_TRY(cudaEventRecord(cx.ev[2 * cx.ev_used], cx.stream));
     }
-    CDMPT_TRY(gemm_oz(N_, N_, N_, X, Y, ep, cx.stream));
+    CDMPT_TRY(gemm_oz(N_, N_, N_, X, Y, ep, cx.stream, nd));
     if (cx.profile) {
         CDMPT_CUDA_TRY(cudaEventRecord(e1, cx.stream));
         ++cx.ev_used;
@@ -1048,7 +1052,7 @@ cdmpt_status Solver<T>::gemm_hp(Context& cx, const OzOperand& X, const OzOperand
     if (cx.st) {
         cx.st->gemm_launches += 1;
         cx.st->gemm_flops += flops;
-        cx.st->tensor_flops += (double)oz_products(kOzDigits) * flops;   // BF16 digit products
+        cx.st->tensor_flops += (double)oz_products(nd) * flops;   // BF16 digit products
     }
     return CDMPT_OK;
 }
@@ -1172,6 +1176,93 @@ cdmpt_status Solver<T>::compute_q(Context& cx) {
     return CDMPT_OK;
 }
 
+// Largest Krylov degree any step's solve needs at relative tolerance tol: the spectrum of A_k
+// lies in [1, 2], on which m CG iterations gain 2 q^m, q = (sqrt(2) - 1) / (sqrt(2) + 1).
+static int krylov_degree(double tol) {
+    return (int)std::ceil(std::log(std::max(tol, 1e-300) / 2.0) / std::log(0.17157));
+}
+
+// The tangent maps take the closed form below unless the products are screened (its factors
+// have other zero patterns than the step's own) or the caller's iteration cap lies below
+// what CG would need: the solves then run and report the cap.
+template <typename T>
+bool Solver<T>::closed_tangent(const cdmpt_opts& o) const {
+    return !(screen_tau_ > 0.f) && krylov_degree(o.cg_tol) <= o.cg_maxit;
+}
+
+// B_k = Z_{k+1} Z_k = 2 (I - A_k^-1), symmetric. An error of B_k is an error of the inverse that
+// every direction of every later step carries on, and the split product has a bias of about
+// -1.5e-7 (tensor-core accumulation truncates): on the mixed precision's 16^3 lattice it alone
+// took the P1 error from 3.1e-7 to 9.2e-7. So the steps that are refined with FP64-class
+// residuals (k >= k_hp) and the two before them (||B|| above about 0.03) form B_k from four
+// Ozaki digits of the pair-stored trajectory (2^-31
+// of the row maxima, ten BF16 products on upper-triangle tiles; the other products of the step
+// keep the split form); the digits of Z_{k+1} serve the next step as those of its Z_k.
+template <typename T>
+cdmpt_status Solver<T>::step_product(Context& cx, int k, int engine) {
+    if constexpr (sizeof(T) == 4) {
+        if (pairs_ && Z_[k].xl && k_hp_ < last_n_ && k >= k_hp_ - 2) {
+            constexpr int nd = 4;
+            for (int j = k; j <= k + 1; ++j) {
+                if (oz_step_[j & 1] == j) continue;
+                CDMPT_TRY(oz_slice(Z_[j].x, Z_[j].xl, N_, N_, ld, oz_[j & 1], cx.stream, nd));
+                oz_step_[j & 1] = j;
+            }
+            OzEpi ep;
+            ep.sym = 2;
+            ep.D = S_.x;
+            ep.ldd = ld;
+            ep.alpha = 1.f;
+            return gemm_hp(cx, oz_[(k + 1) & 1], oz_[k & 1], ep, nd);
+        }
+    }
+    Epilogue<T> ep;
+    ep.sym = true;
+    return gemm(cx, N_, N_, N_, Z_[k + 1].op(), Z_[k].op(), S_.x, ep, nullptr, engine);
+}
+
+// out_d = tangent of step k at dZ_d, for D stacked symmetric directions (both with their TF32
+// split; out is another buffer). From A dZ' = 2 dZ - Z' (Z dZ + dZ Z), Z' = 2 Z V, V = A^-1:
+//   dZ' = 2 V dZ V - 1/2 Z' dZ Z' = 1/4 (U+ dZ U- + U- dZ U+),  U+- = 2 V +- Z',
+// and 2 V = 2 I - Z' Z, so U+- = 2 I + E+-, E+- = +-Z' - Z' Z, from one symmetric product of
+// the trajectory shared by all directions. With G = 2 dZ + dZ E-:
+//   dZ' = sym(G + 1/2 E+ G),
+// two products per direction and no linear solve (the CG form takes three products for the
+// right side and one per iteration, 4 to 9 of them). The terms are corrections to 2 dZ of the
+// size of E+-, so the early steps (||Z|| small) lose no digits. The map is self-adjoint
+// (1/4 (U+ . U- + U- . U+) with symmetric factors), so the reverse sweep uses it too.
+// Scratch: S_, A1_, RHS_, P_.
+template <typename T>
+cdmpt_status Solver<T>::tangent_step(Context& cx, int k, int D, const Buf<T>& in, Buf<T>& out,
+                                     int engine) {
+    const int N = N_, rows = D * N;
+    Buf<T>&Em = A1_, &Ep = RHS_, &G = P_;
+    CDMPT_TRY(step_product(cx, k, engine));
+    // the TF32 engines read only the split of the factors
+    const bool split = engine == CDMPT_GEMM_TC_3XTF32 || engine == CDMPT_GEMM_TC_TF32;
+    CDMPT_TRY(Ew<T>::tangent_factors(split ? nullptr : Em.x, split ? nullptr : Ep.x, Z_[k + 1].x,
+                                     S_.x, blk_, cx.stream, Em.hi, Em.lo, Ep.hi, Ep.lo));
+    {   // G^T = 2 dZ + (dZ E-)^T, block by block
+        Epilogue<T> ep;
+        ep.beta = 2.0;
+        ep.C = in.x;
+        ep.ldc = ld;
+        ep.trans_block = N;
+        ep.Dhi = G.hi;
+        ep.Dlo = G.lo;
+        CDMPT_TRY(gemm(cx, rows, N, N, in.op(), Em.op(), G.x, ep, nullptr, engine));
+    }
+    {   // (G + 1/2 E+ G)^T = G^T + 1/2 G^T E+
+        Epilogue<T> ep;
+        ep.alpha = 0.5;
+        ep.beta = 1.0;
+        ep.C = G.x;
+        ep.ldc = ld;
+        CDMPT_TRY(gemm(cx, rows, N, N, G.op(), Ep.op(), out.x, ep, nullptr, engine));
+    }
+    return Ew<T>::symmetrize(out.x, N, ld, D, cx.stream, out.hi, out.lo);
+}
+
 // Reverse sweep. With Zh_{k+1} the (symmetric) adjoint of Z_{k+1}, the step
 // Z_{k+1} = 2 A_k^-1 Z_k, whose tangent is A_k dZ_{k+1} = 2 dZ_k - (Z_k dZ_k +
 // dZ_k Z_k) Z_{k+1}, gives with V = Zh_{k+1} A_k^-1 (one CG solve)
@@ -1199,8 +1290,23 @@ cdmpt_status Solver<T>::vjp_p0(Context& cx, const double* G0, double* grad, doub
     Buf<T>& VT = Z1b_;
     Buf<T>& M1T = A1_;
     Buf<T>& B = RHS_;
-    for (int k = n - 1; k >= 0; --k) {
-        CDMPT_TRY(need(cx, k));   // checkpointing: each segment recomputed once, last first
+    const bool closed = closed_tangent(o);
+    oz_step_[0] = oz_step_[1] = -1;
+    if (closed) {   // the tangent of a step is self-adjoint: Zh_k = tangent_step(Zh_{k+1})
+        Buf<T>* cur = &Z1a_;
+        Buf<T>* nxt = &Z1b_;
+        CDMPT_TRY(Ew<T>::axpby(cur->x, Zh_.x, blk_, 1.0, 0.0, nullptr, cx.stream, cur->hi,
+                               cur->lo));
+        for (int k = n - 1; k >= 0; --k) {
+            CDMPT_TRY(need(cx, k));   // checkpointing: each segment recomputed once, last first
+            CDMPT_TRY(tangent_step(cx, k, 1, *cur, *nxt, acc));
+            std::swap(cur, nxt);
+        }
+        CDMPT_CUDA_TRY(cudaMemcpyAsync(Zh_.x, cur->x, blk_ * sizeof(T), cudaMemcpyDeviceToDevice,
+                                       cx.stream));
+    }
+    for (int k = n - 1; k >= 0 && !closed; --k) {
+        CDMPT_TRY(need(cx, k));
         CgArgs a;
         a.W = &W_[k];
         a.rhs = Zh_.x;
@@ -1255,6 +1361,10 @@ cdmpt_status Solver<T>::vjp_p0(Context& cx, const double* G0, double* grad, doub
     CDMPT_TRY(Ew<T>::trace(Zh_.x, N, ld, 1, sc_ + S_TRQ + 1, cx.stream));
     CDMPT_TRY(read_scalars(cx, sc_, S_NSLOTS));
     const double trQ = cx.pinned[S_TRQ], trZh = cx.pinned[S_TRQ + 1];
+    if (closed && sizeof(T) == 4 && !std::isfinite(trZh)) {
+        set_error("the adjoint sweep met a non-finite value: no solution of its linear systems");
+        return CDMPT_ERR_CG_MAXITER;
+    }
     const double c = (!gc && trQ > 0) ? last_s2_ * trZh / trQ : 0.0;
     CDMPT_TRY(Ew<T>::lincomb(Zh_.x, Zh_.x, -last_s2_, Qmu_.x, c, blk_, cx.stream));
     // optional + p0_weight P0 = p0_weight (I + Z_n) / 2, added in the padded buffer (the
@@ -1854,6 +1964,7 @@ cdmpt_status Solver<T>::solve(Context& cx, const double* H0, const double* H1, i
             }
         }
         st.fp64_residual_first_step = k_hp;
+        k_hp_ = k_hp;
         // split-TF32 passes until the step residuals settle (one pass from the sweep's
         // trajectory, see refine_settle); from then on (including the Newton steps that
         // follow) every pass forms the residuals of steps k >= k_hp with Ozaki-sliced
@@ -1949,7 +2060,14 @@ cdmpt_status Solver<T>::solve(Context& cx, const double* H0, const double* H1, i
             CDMPT_TRY(Ew<T>::init_z(Z1->x, H1, N, ld, ld, D, -s2, 0.0, cx.stream, Z1->hi,
                                     Z1->lo));
         int total = 0, hint = 1;
-        for (int k = 0; k < n; ++k) {
+        const bool closed = closed_tangent(o);
+        oz_step_[0] = oz_step_[1] = -1;
+        for (int k = 0; k < n && closed; ++k) {
+            CDMPT_TRY(need(cx, k));
+            CDMPT_TRY(tangent_step(cx, k, D, *Z1, *Z1n, acc));
+            std::swap(Z1, Z1n);
+        }
+        for (int k = 0; k < n && !closed; ++k) {
             CDMPT_TRY(need(cx, k));
             {   // S^T = Z1 Z_k (stacked over directions)
                 Epilogue<T> ep;
@@ -2034,6 +2152,10 @@ cdmpt_status Solver<T>::solve(Context& cx, const double* H0, const double* H1, i
         st.trace_Q = trQ;
         for (int d = 0; d < D; ++d) {
             const double trP1 = 0.5 * cx.pinned[S_TRZ1 + d];
+            if (closed && sizeof(T) == 4 && !std::isfinite(trP1)) {
+                set_error("the response met a non-finite value: no solution of its linear systems");
+                return CDMPT_ERR_CG_MAXITER;
+            }
             // grand canonical: mu stays fixed, so mu1 = 0 and P1 = Z1 / 2
             const double mu1 = (!gc && trQ > 0) ? -trP1 / trQ : 0.0;
             if (mu1_out) mu1_out[d] = mu1;

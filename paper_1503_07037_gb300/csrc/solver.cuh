@@ -203,13 +203,22 @@ private:
     // pair-stored trajectory (FP64-class residuals).
     cdmpt_status residual_hp(Context& cx, int k);
     // D = op(X Y^T) by gemm_oz, with the profile events and statistics of gemm()
-    cdmpt_status gemm_hp(Context& cx, const OzOperand& X, const OzOperand& Y, const OzEpi& ep);
+    cdmpt_status gemm_hp(Context& cx, const OzOperand& X, const OzOperand& Y, const OzEpi& ep,
+                         int nd = kOzDigits);
     // Z_k += d, symmetrised (pair storage: without rounding the sum to FP32)
     cdmpt_status correct(Context& cx, int k, const T* d);
     // Z_0 += shift I
     cdmpt_status shift_z0(Context& cx, double shift);
     // P0 = (I + Z_n)/2 of the last solve in FP64 (device, leading dimension ldo)
     cdmpt_status p0_out(Context& cx, double* out, int ldo);
+    // Tangent of step k applied to D stacked directions (response, adjoint), closed form.
+    bool closed_tangent(const cdmpt_opts& o) const;
+    cdmpt_status tangent_step(Context& cx, int k, int D, const Buf<T>& in, Buf<T>& out,
+                              int engine);
+    // B_k = Z_{k+1} Z_k into S_.x (symmetric): I - B_k / 2 is the inverse of A_k
+    cdmpt_status step_product(Context& cx, int k, int engine);
+    int oz_step_[2] = {-1, -1};      // steps whose Z_k digits oz_[0], oz_[1] hold (step_product)
+    int k_hp_ = 0;                   // first step of the FP64-class residuals of the last solve
     cdmpt_status occupation(Context& cx, int n, double* trP, double* zz);
     cdmpt_status compute_q(Context& cx);
     cdmpt_status read_scalars(Context& cx, const double* dev, int count);

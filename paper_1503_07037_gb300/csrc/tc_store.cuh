@@ -125,6 +125,58 @@ __device__ __forceinline__ float epi_block32_plain(const EpiParams<float>& p, in
     return local;
 }
 
+// Transposed placement (never symmetric): element (m, n) of the product goes to row
+// trans_block b + n, column m - trans_block b of its row block b, so that the 32 lanes (rows)
+// write consecutive columns. The loads of eight columns are issued before their stores: an
+// element-wise loop waits one memory latency per column for C, 32 per block.
+template <bool SPLIT>
+__device__ __forceinline__ float epi_block32_trans(const EpiParams<float>& p, int m0, int n,
+                                                   const float* S, int lane) {
+    constexpr int RB = 8;
+    const int m = m0 + lane, N = p.N;
+    const bool row_ok = m < p.M;
+    const int b = m / p.trans_block;
+    const size_t r0 = (size_t)b * p.trans_block + n, c = (size_t)(m - b * p.trans_block);
+    const size_t ldd = (size_t)p.ldd, ldc = (size_t)p.ldc, lde = (size_t)p.lde;
+    float* const D = p.D;
+    float* const Dhi = p.Dhi;
+    float* const Dlo = p.Dlo;
+    const float alpha = p.alpha, beta = p.beta, gamma = p.gamma;
+    const bool has_c = beta != 0.f, has_g = gamma != 0.f, has_dot = p.dot != nullptr;
+    const bool has_e = has_dot && p.E != nullptr;
+    const int md = has_g ? m % p.diag_block : -1;
+    float local = 0.f;
+#pragma unroll 1
+    for (int j0 = 0; j0 < 32; j0 += RB) {
+        float cv[RB], ev[RB];
+#pragma unroll
+        for (int i = 0; i < RB; ++i) {
+            const bool ok = row_ok && n + j0 + i < N;
+            cv[i] = (ok && has_c) ? p.C[(r0 + j0 + i) * ldc + c] : 0.f;
+            ev[i] = (ok && has_e) ? p.E[(r0 + j0 + i) * lde + c] : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < RB; ++i) {
+            const bool ok = row_ok && n + j0 + i < N;
+            float v = alpha * S[lane * 33 + j0 + i];
+            v = has_c ? fmaf(beta, cv[i], v) : v;
+            v = md == n + j0 + i ? v + gamma : v;
+            const size_t o = (r0 + j0 + i) * ldd + c;
+            if (ok) D[o] = v;
+            if constexpr (SPLIT) {
+                float h, l;
+                split_tf32(v, h, l);
+                if (ok) {
+                    Dhi[o] = h;
+                    Dlo[o] = l;
+                }
+            }
+            local += (ok && has_dot) ? v * (has_e ? ev[i] : v) : 0.f;
+        }
+    }
+    return local;
+}
+
 // Applies the epilogue (alpha, beta C, gamma I, transposed placement, TF32 split copies,
 // symmetric mirror, Frobenius dot; the same arithmetic as epi_apply and epi_apply_sym) to
 // the block of an output tile with rows m0 .. m0 + 31 and columns n .. n + 31. Lane l holds
@@ -137,11 +189,8 @@ __device__ __forceinline__ float epi_block32(const EpiParams<float>& p, int m0, 
     float local = 0.f;
     xpose_in(a, S, lane);
     if (p.trans_block > 0) {
-        // transposed placement (never symmetric): element by element, lane = row
-#pragma unroll 1
-        for (int j = 0; j < 32; ++j)
-            if (m0 + lane < p.M && n + j < p.N)
-                local += epi_apply(p, m0 + lane, n + j, S[lane * 33 + j]);
+        local = p.Dhi ? epi_block32_trans<true>(p, m0, n, S, lane)
+                      : epi_block32_trans<false>(p, m0, n, S, lane);
         __syncwarp();
         return local;
     }
