@@ -274,6 +274,47 @@ __global__ void k_lincomb(T* __restrict__ out, const T* X, double a, const T* Y,
     }
 }
 
+// The coefficient blocks of a matrix polynomial in one pass over the powers of S = W - c I.
+// NP: powers read (W, S^2 .. S^NP), NB: blocks written, the last one with its TF32 split.
+// Bound by memory: NP reads and NB + 2 writes of N x ld floats, against NP - 1 + NB symmetric
+// products; one axpby pass per coefficient would move three arrays for each of NB (NP + 1).
+template <typename T, int NP, int NB>
+__global__ void k_poly_blocks(typename Ew<T>::PolyBlocks p, double c, int N, int ld,
+                              size_t nvec) {
+    constexpr int W = Vec<T>::W;
+    T k[NB][NP + 1];
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int j = 0; j <= NP; ++j) k[b][j] = (T)p.coef[b][j];
+    const T tc = (T)c;
+    const size_t lv = (size_t)ld / W;
+    for (size_t v = blockIdx.x * (size_t)blockDim.x + threadIdx.x; v < nvec;
+         v += (size_t)gridDim.x * blockDim.x) {
+        const size_t r = v / lv;
+        const int d = (int)r - (int)(v - r * lv) * W;   // diagonal position inside the vector
+        T x[NP][W];
+#pragma unroll
+        for (int j = 0; j < NP; ++j) load16(p.P[j] + v * W, x[j]);
+#pragma unroll
+        for (int i = 0; i < W; ++i)
+            if (d == i) x[0][i] -= tc;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            T y[W];
+#pragma unroll
+            for (int i = 0; i < W; ++i) {
+                y[i] = k[b][1] * x[0][i];
+#pragma unroll
+                for (int j = 1; j < NP; ++j) y[i] = fma(k[b][j + 1], x[j][i], y[i]);
+                if (d == i) y[i] += k[b][0];
+            }
+            store16(p.out[b] + v * W, y);
+            if (b == NB - 1) put_split16(p.hi, p.lo, v * W, y);
+        }
+    }
+}
+
 // Em = -Y - B, Ep = Y - B: the factors of a step's tangent map, both with their TF32 split, in
 // one pass over Y and B. Bound by memory: 2 reads and 6 writes of N x ld floats (2 and 2 of
 // doubles); the split products that read the result (hi, lo) leave no use for Em, Ep themselves
@@ -701,6 +742,29 @@ cdmpt_status Ew<T>::lincomb(T* out, const T* X, double a, const T* Y, double b, 
                             cudaStream_t s) {
     const size_t nvec = count / Vec<T>::W;
     k_lincomb<T><<<grid_for(nvec), kThreads, 0, s>>>(out, X, a, Y, b, nvec);
+    LAUNCH_CHECK();
+    return CDMPT_OK;
+}
+
+template <typename T>
+cdmpt_status Ew<T>::poly_blocks(const PolyBlocks& p, double c, int N, int ld, cudaStream_t s) {
+    const size_t nvec = (size_t)N * ld / Vec<T>::W;
+    const int g = grid_for(nvec);
+    auto is = [&](int np, int nb) { return p.np == np && p.nb == nb; };
+    if (is(2, 1))
+        k_poly_blocks<T, 2, 1><<<g, kThreads, 0, s>>>(p, c, N, ld, nvec);
+    else if (is(3, 3))
+        k_poly_blocks<T, 3, 3><<<g, kThreads, 0, s>>>(p, c, N, ld, nvec);
+    else if (is(3, 4))
+        k_poly_blocks<T, 3, 4><<<g, kThreads, 0, s>>>(p, c, N, ld, nvec);
+    else if (is(4, 4))
+        k_poly_blocks<T, 4, 4><<<g, kThreads, 0, s>>>(p, c, N, ld, nvec);
+    else if (is(5, 4))
+        k_poly_blocks<T, 5, 4><<<g, kThreads, 0, s>>>(p, c, N, ld, nvec);
+    else {
+        set_error("matrix polynomial: no kernel for this block shape");
+        return CDMPT_ERR_ARG;
+    }
     LAUNCH_CHECK();
     return CDMPT_OK;
 }

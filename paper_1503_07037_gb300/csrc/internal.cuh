@@ -181,6 +181,18 @@ struct Ew {
                                  T* hi = nullptr, T* lo = nullptr);
     static cdmpt_status lincomb(T* out, const T* X, double a, const T* Y, double b, size_t count,
                                 cudaStream_t s);
+    // Blocks of a matrix polynomial in S = P[0] - c I (P[j] = S^(j+1) for j >= 1): for b < nb,
+    // out[b] = sum_{j <= np} coef[b][j] S^j, the last block with its split (hi, lo). Elementwise:
+    // an output may be one of the inputs.
+    struct PolyBlocks {
+        const T* P[5] = {};
+        T* out[5] = {};
+        double coef[5][6] = {};
+        int np = 0, nb = 0;
+        T* hi = nullptr;
+        T* lo = nullptr;
+    };
+    static cdmpt_status poly_blocks(const PolyBlocks& b, double c, int N, int ld, cudaStream_t s);
     // The right and left factors of a step's tangent map: Em = -Y - B, Ep = Y - B, with splits.
     static cdmpt_status tangent_factors(T* Em, T* Ep, const T* Y, const T* B, size_t count,
                                         cudaStream_t s, T* Em_hi, T* Em_lo, T* Ep_hi, T* Ep_lo);

@@ -15,6 +15,11 @@
 // in their own exponent range instead of rounding them against I or 2 Z_k,
 // which makes the CG result about three times more accurate than solving for
 // Z_{k+1} against A_k = I + Z_k^2 directly.
+// Everything of order 0 is a function of H0 and commutes, and the spectrum of W_k lies in
+// [0, b_k^2] with b_k known from the Gershgorin interval, so the sweeps need no CG: a polynomial
+// in W_k of the degree that the interval and the tolerance ask for gives Z_{k+1} from a few
+// symmetric products (step0). CG stays for the solves without such a bound or symmetry and
+// for screened products.
 //
 // First-order maps (response, adjoint): with V_k = A_k^-1 the step Z_{k+1} = 2 Z_k V_k has the
 // tangent dZ_{k+1} = 2 V_k dZ_k V_k - 1/2 Z_{k+1} dZ_k Z_{k+1} (see tangent_step), and
@@ -820,6 +825,134 @@ cdmpt_status Solver<T>::tanh_taylor(Context& cx, int m) {
     return CDMPT_OK;
 }
 
+// The polynomial is the Chebyshev series of 1 / (x0 + w) on [lo, hi], with t = S / h in [-1, 1],
+// h = (hi - lo) / 2, c = (hi + lo) / 2, A = x0 + c:
+//   1 / (A + h t) = (1 / g) [1 + 2 sum_{j >= 1} (-q)^j T_j(t)],  g = sqrt(A^2 - h^2), q = h / (A + g),
+// cut after degree m with an error below 2 q^(m+1) / (g (1 - q)); near-minimax. For [0, 1]
+// and x0 = 1, q = 0.17: degree 9 for 1e-7, 18 for 1e-14. The shapes (s, r) below are the ones
+// with the fewest products s - 1 + r for their degree; a shape's whole degree is used.
+bool InversePoly::fit(double x0, double lo, double hi, double tol, int max_degree) {
+    static const int shape[][2] = {{1, 0}, {2, 0}, {2, 1}, {2, 2}, {3, 2}, {3, 3}, {4, 3}, {5, 3}};
+    s = r = 0;
+    const double h = 0.5 * (hi - lo), A = x0 + 0.5 * (hi + lo);
+    c = 0.5 * (hi + lo);
+    if (!(h > 0.0) || !(A > h) || !(tol > 0.0)) return false;
+    const double g = std::sqrt((A - h) * (A + h)), q = h / (A + g);
+    double err = (x0 + hi) * 2.0 * q / (g * (1.0 - q));   // degree 0
+    for (need = 0; err > tol; ++need) {
+        if (need >= max_degree) return false;
+        err *= q;
+    }
+    for (const auto& sh : shape)
+        if (sh[0] * (sh[1] + 1) >= need && sh[0] * (sh[1] + 1) <= kMaxDegree) {
+            s = sh[0];
+            r = sh[1];
+            break;
+        }
+    if (s == 0 || degree() > std::max(max_degree, 1)) {
+        s = 0;
+        return false;
+    }
+    // Chebyshev to monomials in t, then powers of S
+    const int m = degree();
+    double t0[kMaxDegree + 1] = {1.0}, t1[kMaxDegree + 1] = {0.0, 1.0}, t2[kMaxDegree + 1];
+    for (int j = 0; j <= m; ++j) a[j] = 0.0;
+    a[0] = 1.0;
+    double f = 2.0;
+    for (int j = 1; j <= m; ++j) {
+        f *= -q;
+        for (int i = 0; i <= j; ++i) a[i] += f * t1[i];
+        for (int i = 0; i <= m; ++i) t2[i] = (i > 0 ? 2.0 * t1[i - 1] : 0.0) - t0[i];
+        for (int i = 0; i <= m; ++i) {
+            t0[i] = t1[i];
+            t1[i] = t2[i];
+        }
+    }
+    double hp = 1.0;
+    for (int j = 0; j <= m; ++j, hp *= h) a[j] /= g * hp;
+    return true;
+}
+
+template <typename T>
+cdmpt_status Solver<T>::poly_eval(Context& cx, const Buf<T>& W, const InversePoly& p,
+                                  double shift, int engine, const Buf<T>** out) {
+    const int N = N_, s = p.s, r = p.r;
+    // C-terms reach the diagonal through gamma: a c-shift of S costs no extra pass
+    auto product = [&](const Buf<T>& X, const Buf<T>& Y, Buf<T>& D, double alpha, double beta,
+                       const Buf<T>* C, double gamma, bool split) -> cdmpt_status {
+        Epilogue<T> ep;
+        ep.alpha = alpha;
+        ep.beta = beta;
+        ep.C = C ? C->x : nullptr;
+        ep.ldc = ld;
+        ep.gamma = gamma;
+        ep.sym = true;
+        if (split) {
+            ep.Dhi = D.hi;
+            ep.Dlo = D.lo;
+        }
+        return gemm(cx, N, N, N, X.op(), Y.op(), D.x, ep, nullptr, engine);
+    };
+    if (s == 2 && r == 0) {   // a2 S^2 + a1 S + a0 in one product of W
+        const double b1 = p.a[1] - 2.0 * p.c * p.a[2];
+        const double b0 = (p.a[0] - shift) - p.a[1] * p.c + p.a[2] * p.c * p.c;
+        CDMPT_TRY(product(W, W, A1_, p.a[2], b1, &W, b0, true));
+        *out = &A1_;
+        return CDMPT_OK;
+    }
+    // powers: S^2 = W^2 - 2 c W + c^2 I, S^3 = S^2 W - c S^2, S^4 = S^2 S^2, S^5 = S^4 W - c S^4.
+    // Only S^2 (or S^4) and S^s are operands and need a split
+    Buf<T>* pw[5] = {nullptr, &A1_, nullptr, nullptr, nullptr};
+    Buf<T>* free_plain[3] = {&S_, &Q_, &R_};
+    int nfree = 3;
+    for (int j = 2; j < s; ++j) pw[j] = j == s - 1 ? &RHS_ : free_plain[--nfree];
+    CDMPT_TRY(product(W, W, *pw[1], 1.0, -2.0 * p.c, &W, p.c * p.c, true));
+    for (int j = 2; j < s; ++j) {
+        if (j == 3)
+            CDMPT_TRY(product(*pw[1], *pw[1], *pw[3], 1.0, 0.0, nullptr, 0.0, s == 4));
+        else
+            CDMPT_TRY(product(*pw[j - 1], W, *pw[j], 1.0, -p.c, pw[j - 1], 0.0, j == s - 1));
+    }
+    // coefficient blocks: the top one (with S^s) starts the Horner scheme in P_
+    typename Ew<T>::PolyBlocks pb;
+    pb.np = s;
+    pb.P[0] = W.x;
+    for (int j = 1; j < s; ++j) pb.P[j] = pw[j]->x;
+    T* low[4] = {};
+    if (s > 2) {   // s = 2: the lower blocks a S + a' I are C-terms of W itself
+        pb.nb = r + 1;
+        int next = 2;   // S^3 .. S^(s-1) end with the blocks: their buffers take outputs
+        for (int b = 0; b < r; ++b) {
+            low[b] = nfree > 0 ? free_plain[--nfree]->x : pw[next++]->x;
+            pb.out[b] = low[b];
+            for (int j = 0; j < s; ++j) pb.coef[b][j] = p.a[b * s + j];
+        }
+        pb.coef[0][0] -= shift;
+    } else {
+        pb.nb = 1;
+    }
+    pb.out[pb.nb - 1] = P_.x;
+    for (int j = 0; j <= s; ++j) pb.coef[pb.nb - 1][j] = p.a[r * s + j];
+    pb.hi = P_.hi;
+    pb.lo = P_.lo;
+    CDMPT_TRY(Ew<T>::poly_blocks(pb, p.c, N, ld, cx.stream));
+    Buf<T>* H = &P_;
+    Buf<T>* Hn = s == 2 ? &RHS_ : &A1_;   // S^2 is not needed any more unless it is S^s
+    for (int b = r - 1; b >= 0; --b) {
+        if (s == 2) {
+            const double a0 = p.a[2 * b] - (b == 0 ? shift : 0.0), a1 = p.a[2 * b + 1];
+            CDMPT_TRY(product(*H, *pw[1], *Hn, 1.0, a1, &W, a0 - a1 * p.c, true));
+        } else {
+            Buf<T> C;
+            C.x = low[b];
+            CDMPT_TRY(product(*H, *pw[s - 1], *Hn, 1.0, 1.0, &C, 0.0, true));
+        }
+        std::swap(H, Hn);
+    }
+    *out = H;
+    return CDMPT_OK;
+}
+
 // One step of the 0th-order recursion: W_k = Z_k Z_k and the correction d of
 // d (I + W_k) = -2 Z_k W_k, then Z_{k+1} = sym(2 Z_k + d) with its TF32 split.
 template <typename T>
@@ -833,6 +966,40 @@ cdmpt_status Solver<T>::step0(Context& cx, int k, int engine, double tol, int ma
         CDMPT_TRY(gemm(cx, N_, N_, N_, Z_[k].op(), Z_[k].op(), W_[k].x, ep, nullptr, engine));
     }
     if (!solve) return CDMPT_OK;
+    // Polynomial form: Z_{k+1} = 2 Z_k p(W_k) = 2 Z_k + 2 Z_k (p(W_k) - I), the correction formed by
+    // itself so that a small W_k keeps its own exponent range. Every product is symmetric and
+    // mirrored (half the tiles of the CG products), there are no vector updates and no scalar is
+    // read back: a saturated step takes W and five products at half tiles in FP32 where CG
+    // took two and about nine whole ones (16^3 lattice, beta 80, FP32: solve 147 -> 70 ms, P1
+    // error 3.5e-6 -> 1.9e-6; N = 2048 in FP64 570 -> 262 ms). Not for BF16 operands (their rounding would pass through several products in a
+    // row) and screened products; a caller's cap on iterations caps the degree as well.
+    const double zb = zbound_[k];
+    InversePoly p;
+    if (!(screen_tau_ > 0.f) && engine != CDMPT_GEMM_TC_BF16 &&
+        p.fit(1.0, 0.0, zb * zb, 0.5 * tol, std::min(maxit, sizeof(T) == 8 ? 20 : 16))) {
+        Epilogue<T> ep;
+        ep.beta = 2.0;
+        ep.C = Z_[k].x;
+        ep.ldc = ld;
+        ep.Dhi = Z_[k + 1].hi;
+        ep.Dlo = Z_[k + 1].lo;
+        ep.sym = true;
+        const Buf<T>* E = &W_[k];
+        if (p.degree() == 1)   // p = 1 - a w with |p - 1 / (1 + w)| level at both ends
+            ep.alpha = -2.0 * (1.0 - 0.8284 * zb * zb);
+        else {
+            ep.alpha = 2.0;
+            CDMPT_TRY(poly_eval(cx, W_[k], p, 1.0, engine, &E));
+        }
+        CDMPT_TRY(gemm(cx, N_, N_, N_, Z_[k].op(), E->op(), Z_[k + 1].x, ep, nullptr, engine));
+        if (engine == CDMPT_GEMM_SIMT || sizeof(T) == 8)   // full tiles, not mirrored
+            CDMPT_TRY(Ew<T>::symmetrize(Z_[k + 1].x, N_, ld, 1, cx.stream, Z_[k + 1].hi,
+                                        Z_[k + 1].lo));
+        *iters += p.degree();
+        if (Z_[k + 1].xl)
+            CDMPT_CUDA_TRY(cudaMemsetAsync(Z_[k + 1].xl, 0, blk_ * sizeof(T), cx.stream));
+        return CDMPT_OK;
+    }
     {   // right side of the correction: -2 Z_k W_k = -2 Z_k^3 (symmetric)
         Epilogue<T> ep;
         ep.alpha = -2.0;
@@ -877,7 +1044,17 @@ template <typename T>
 cdmpt_status Solver<T>::sweep(Context& cx, const double* H0, double mu, double s2,
                               const cdmpt_opts& o, int n, int engine, double tol,
                               int* cg_iters) {
-    CDMPT_TRY(init_z0(cx, H0, mu, s2, s2 * std::max(gmax_ - mu, mu - gmin_), acc_cur_));
+    const double rho = s2 * std::max(gmax_ - mu, mu - gmin_);
+    CDMPT_TRY(init_z0(cx, H0, mu, s2, rho, acc_cur_));
+    // |Z_k| <= tanh(2^k atanh |Z_0|), with a margin for the rounding of the products
+    zbound_.assign(n + 1, 0.0);
+    double zb = fdx_ ? std::tanh(rho) : rho;
+    const double margin = engine == CDMPT_GEMM_TC_TF32 ? 1e-3 : 1e-6;
+    for (int k = 0; k <= n; ++k) {
+        zb = std::min(zb * (1.0 + margin), 1.0);
+        zbound_[k] = zb;
+        zb = 2.0 * zb / (1.0 + zb * zb);
+    }
     int total = 0, hint = 1;
     for (int k = 0; k < n; ++k)
         CDMPT_TRY(step0(cx, k, engine, tol, o.cg_maxit, true, true, &hint, &total));

@@ -58,6 +58,21 @@ struct Buf {
     }
 };
 
+// Polynomial p(S) = sum_j a[j] S^j in S = W - c I that approximates (x0 I + W)^-1 for symmetric W
+// with spectrum in [lo, hi], evaluated with s - 1 products for the powers S^2 .. S^s and r Horner
+// products over blocks of s coefficients (degree up to s (r + 1)).
+struct InversePoly {
+    static constexpr int kMaxDegree = 20;
+    int s = 0, r = 0;      // s = 0: no polynomial
+    int need = 0;          // smallest degree that meets the tolerance
+    double c = 0.0;
+    double a[kMaxDegree + 1] = {};
+    int degree() const { return s * (r + 1); }
+    // Relative error (x0 + w) |p - 1 / (x0 + w)| <= tol on [lo, hi], degree <= max_degree;
+    // false (s = 0) if that takes a higher degree
+    bool fit(double x0, double lo, double hi, double tol, int max_degree);
+};
+
 template <typename T>
 class Solver {
 public:
@@ -215,6 +230,12 @@ private:
     bool closed_tangent(const cdmpt_opts& o) const;
     cdmpt_status tangent_step(Context& cx, int k, int D, const Buf<T>& in, Buf<T>& out,
                               int engine);
+    // E = p(W - c I) - shift I for a polynomial of degree >= 2, by products on upper-triangle
+    // tiles; *out is one of the scratch buffers (with its split). Scratch: A1_, RHS_, P_, R_,
+    // Q_, S_.
+    cdmpt_status poly_eval(Context& cx, const Buf<T>& W, const InversePoly& p, double shift,
+                           int engine, const Buf<T>** out);
+    std::vector<double> zbound_;     // bound of |Z_k| of the running (last) sweep, k = 0 .. n
     // B_k = Z_{k+1} Z_k into S_.x (symmetric): I - B_k / 2 is the inverse of A_k
     cdmpt_status step_product(Context& cx, int k, int engine);
     int oz_step_[2] = {-1, -1};      // steps whose Z_k digits oz_[0], oz_[1] hold (step_product)
