@@ -18,9 +18,16 @@
 // integers (K <= 16384 keeps those below 2^31). The groups g = 4, 5, 6 weigh 2^-32 and less
 // of the leading one and accumulate over the whole K in TMEM; the truncating FP32 accumulation
 // leaves them an error near 2^-47 of the leading term at K = 8192. The epilogue forms
-//   2^(e_i + f_j - 38) [G_0 2^24 + G_1 2^16 + G_2 2^8 + G_3 + g_4 2^-8 + g_5 2^-16 + g_6 2^-24]
-// from the 64-bit integer part and the FP32 tail in FP64, then the epilogue of the other
-// engines (alpha, beta C, gamma on the diagonal blocks, transposed placement, fused dot).
+//   2^(e_i + f_j - 62) [G_0 2^48 + G_1 2^40 + G_2 2^32 + G_3 2^24 + g_4 2^16 + g_5 2^8 + g_6]
+// as a 128-bit integer and rounds it once to FP64 by integer operations, then the epilogue of
+// the other engines (alpha, beta C, gamma on the diagonal blocks, transposed placement, fused
+// dot). The FP64 pipe of this part runs two operations per clock and SM: about 14 FP64
+// operations per element (conversions, sums, ldexp) held a 256 x 64 tile's epilogue to 29 us,
+// as long as a third of the MMAs of K = 2048 and most of a small product; the integer form
+// leaves one for beta C and one for the dot, and a power-of-two alpha goes into the exponent.
+//
+// Symmetric results (ep.sym: W = Z Z, functions of one matrix) compute the tiles that meet the
+// upper triangle, about N^2 / 2 of the elements, and store every element n > m twice.
 //
 // Kernel (k_gemm_oz64): a cluster of two CTAs per 256 x 64 output tile
 // (tcgen05.mma.cta_group::2.kind::f16, M = 256, N = 64: seven 64-column accumulators fit the
@@ -38,6 +45,7 @@
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 
+#include <cmath>
 #include <cstdlib>
 #include <cstring>
 #include <string>
@@ -219,10 +227,66 @@ __device__ __forceinline__ void st8(uint32_t ta, const int* v) {
                  : "memory");
 }
 
+// FP64 value of (J 2^16 + T) 2^e, rounded to nearest even. Integer operations only, but for
+// results outside the normal range.
+__device__ __forceinline__ double oz64_value(long long J, long long T, int e) {
+    unsigned long long lo = (unsigned long long)J << 16;
+    long long hi = J >> 48;
+    const unsigned long long sum = lo + (unsigned long long)T;
+    hi += (T >> 63) + (sum < lo ? 1 : 0);
+    lo = sum;
+    const bool neg = hi < 0;
+    if (neg) {
+        lo = 0ull - lo;
+        hi = ~hi + (lo == 0ull ? 1 : 0);
+    }
+    unsigned long long h = (unsigned long long)hi;
+    if ((h | lo) == 0ull) return 0.0;
+    int lz;
+    if (h == 0ull) {
+        const int l = __clzll((long long)lo);
+        h = lo << l;
+        lo = 0ull;
+        lz = 64 + l;
+    } else {
+        lz = __clzll((long long)h);
+        if (lz > 0) {
+            h = (h << lz) | (lo >> (64 - lz));
+            lo <<= lz;
+        }
+    }
+    unsigned long long m = h >> 11;   // 53 bits, the leading one at bit 52
+    const unsigned long long rest = h & 0x7ffull;
+    if (rest > 0x400ull || (rest == 0x400ull && (lo != 0ull || (m & 1ull)))) ++m;
+    const int be = 1023 + 127 - lz + e;
+    if (be >= 1 && be <= 2045) {
+        const unsigned long long b = ((unsigned long long)be << 52) + (m - (1ull << 52)) +
+                                     (neg ? 1ull << 63 : 0ull);
+        return __longlong_as_double((long long)b);
+    }
+    const double v = ldexp((double)m, 75 - lz + e);
+    return neg ? -v : v;
+}
+
+// Tile t of a launch: row-tile fastest, or, for a symmetric result, over the tiles whose 64
+// columns reach row 256 mt: column tile nt has nt / 4 + 1 of them, 2 a (a + 1) before nt = 4 a.
+__device__ __forceinline__ void oz64_tile(int t, int num_mt, bool sym, int* mt, int* nt) {
+    if (!sym) {
+        *mt = t % num_mt;
+        *nt = t / num_mt;
+        return;
+    }
+    int a = 0;
+    while (2 * (a + 1) * (a + 2) <= t) ++a;
+    const int rem = t - 2 * a * (a + 1);
+    *nt = 4 * a + rem / (a + 1);
+    *mt = rem % (a + 1);
+}
+
 __global__ void __launch_bounds__(Z_THREADS, 1)
     k_gemm_oz64(const __grid_constant__ Oz64Maps maps, const __grid_constant__ EpiParams<double> p,
                 const int* __restrict__ ex_, const int* __restrict__ ey_, int K, int num_mt,
-                int total_tiles, const double* skip, int* err) {
+                int total_tiles, int alpha_exp, int alpha_neg, const double* skip, int* err) {
     if (skip != nullptr && *skip != 0.0) return;   // both CTAs of a pair read the same flag
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -280,7 +344,8 @@ __global__ void __launch_bounds__(Z_THREADS, 1)
             uint32_t it = 0;
             bool ok = true;
             for (int t = cid; t < total_tiles && ok; t += ncl) {
-                const int mt = t % num_mt, nt = t / num_mt;
+                int mt, nt;
+                oz64_tile(t, num_mt, p.sym != 0, &mt, &nt);
                 const int m0 = mt * (2 * BM) + (int)rank * BM;
                 const int y0 = nt * Z_BN + (int)rank * (Z_BN / 2);
                 for (int kb = 0; kb < num_k; ++kb, ++it) {
@@ -382,7 +447,8 @@ __global__ void __launch_bounds__(Z_THREADS, 1)
         uint32_t gc = 0, tc = 0;
         double dsum = 0.0;
         for (int t = cid; t < total_tiles; t += ncl, ++tc) {
-            const int mt = t % num_mt, nt = t / num_mt;
+            int mt, nt;
+            oz64_tile(t, num_mt, p.sym != 0, &mt, &nt);
             const int m = mt * (2 * BM) + (int)rank * BM + 32 * q + lane;
             const int n0 = nt * Z_BN + Z_CW * h;
             int G[Z_NX][Z_CW];
@@ -446,7 +512,7 @@ __global__ void __launch_bounds__(Z_THREADS, 1)
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         const int n = n0 + c0 + j;
-                        const bool ok = n < p.N;
+                        const bool ok = n < p.N && !(p.sym && n < m);
                         size_t rr, cc;
                         epi_position(p, m, n, rr, cc);
                         eyv[j] = ok ? ey_[n] : 0;
@@ -456,23 +522,24 @@ __global__ void __launch_bounds__(Z_THREADS, 1)
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         const int n = n0 + c0 + j;
-                        if (n < p.N) {
-                            long long I = 0;
+                        if (n < p.N && !(p.sym && n < m)) {
+                            long long J = 0;
 #pragma unroll
-                            for (int g = 0; g < Z_NX; ++g) I = I * 256 + (long long)(int)r[g][j];
-                            const double tail =
-                                (double)__uint_as_float(r[Z_NX][j]) * (1.0 / 256.0) +
-                                (double)__uint_as_float(r[Z_NX + 1][j]) * (1.0 / 65536.0) +
-                                (double)__uint_as_float(r[Z_NX + 2][j]) * (1.0 / 16777216.0);
-                            const double acc =
-                                ldexp((double)I + tail, ex + eyv[j] - 14 - 8 * (Z_NX - 1));
+                            for (int g = 0; g < Z_NX; ++g) J = J * 256 + (long long)(int)r[g][j];
+                            J = J * 256 + (long long)__float2int_rn(__uint_as_float(r[Z_NX][j]));
+                            const long long T =
+                                (long long)__float2int_rn(__uint_as_float(r[Z_NX + 1][j])) * 256 +
+                                (long long)__float2int_rn(__uint_as_float(r[Z_NX + 2][j]));
+                            double v = oz64_value(J, T, ex + eyv[j] + alpha_exp - 62);
+                            v = alpha_neg < 0 ? p.alpha * v : (alpha_neg ? -v : v);
                             size_t rr, cc;
                             epi_position(p, m, n, rr, cc);
-                            double v = p.alpha * acc;
                             if (p.beta != 0.0) v = fma(p.beta, cv[j], v);
                             if (p.gamma != 0.0 && (m % p.diag_block) == n) v += p.gamma;
                             p.D[rr * p.ldd + cc] = v;
-                            if (p.dot) dsum += v * (p.E ? ev[j] : v);
+                            const bool mirror = p.sym && n != m;
+                            if (mirror) p.D[(size_t)n * p.ldd + m] = v;
+                            if (p.dot) dsum += v * (p.E ? ev[j] : v) * (mirror ? 2.0 : 1.0);
                         }
                     }
                 }
@@ -504,43 +571,107 @@ __global__ void __launch_bounds__(Z_THREADS, 1)
     }
 }
 
-// One warp per row: the row's power of two and the seven BF16 digits of every element
-// (zeros in the padding columns cols .. ld - 1).
-__global__ void k_oz64_slice(const double* __restrict__ x, int rows, int cols, int ld,
-                             Oz64Operand out, const double* skip) {
+// The 55-bit integer round(x 2^(55 - e)) of a double's bits in a row whose largest biased
+// exponent is emax >= 1 (e = emax - 1022); ties to even.
+__device__ __forceinline__ long long oz64_fixed(unsigned long long b, int emax) {
+    const int eb = (int)(b >> 52) & 0x7ff;
+    unsigned long long M = b & 0xfffffffffffffull;
+    if (eb) M |= 1ull << 52;
+    const int sh = (eb ? eb : 1) - emax + 2;
+    unsigned long long t;
+    if (sh >= 0) {
+        t = M << sh;
+    } else if (sh > -55) {
+        const unsigned long long half = 1ull << (-sh - 1), rest = M & (2ull * half - 1ull);
+        t = M >> -sh;
+        if (rest > half || (rest == half && (t & 1ull))) ++t;
+    } else {
+        t = 0ull;
+    }
+    return (b >> 63) ? -(long long)t : (long long)t;
+}
+
+// One block per row: the row's power of two and the seven BF16 digits of every element (zeros
+// in the padding columns cols .. ld - 1). Bound by memory (8 bytes in, 14 out, per element):
+// the exponent and the fixed-point value come from the bits of the double, since frexp,
+// ldexp and the conversion are FP64-pipe operations at two per clock and SM; four columns per
+// thread, so that a warp writes 256 bytes of each digit array at a time.
+constexpr int Z_SLICE_THREADS = 128;
+__global__ void __launch_bounds__(Z_SLICE_THREADS)
+    k_oz64_slice(const double* __restrict__ x, int rows, int cols, int ld, Oz64Operand out,
+                 const double* skip) {
     if (skip != nullptr && *skip != 0.0) return;
-    constexpr int BITS = 8 * Z_ND - 1;   // 55
-    const int lane = threadIdx.x & 31;
-    const int wpb = blockDim.x >> 5;
-    for (int r = blockIdx.x * wpb + (threadIdx.x >> 5); r < rows; r += gridDim.x * wpb) {
+    __shared__ int wmax[Z_SLICE_THREADS / 32];
+    const bool vec = (((uintptr_t)x | ((uintptr_t)ld * 8)) & 15) == 0;
+    const int ncol = out.ld;   // a multiple of 8
+    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
         const double* xr = x + (size_t)r * ld;
-        double mx = 0.0;
-        for (int j = lane; j < cols; j += 32) mx = fmax(mx, fabs(xr[j]));
+        auto load4 = [&](int j, unsigned long long (&b)[4]) {
+            if (vec && j + 4 <= cols) {
+                const ulonglong2 u = *(const ulonglong2*)(xr + j);
+                const ulonglong2 w = *(const ulonglong2*)(xr + j + 2);
+                b[0] = u.x;
+                b[1] = u.y;
+                b[2] = w.x;
+                b[3] = w.y;
+            } else {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        int e = 0;
-        if (mx > 0.0) (void)frexp(mx, &e);   // mx = m 2^e, m in [0.5, 1): |x| 2^-e < 1
-        if (lane == 0) out.e[r] = e;
+                for (int i = 0; i < 4; ++i)
+                    b[i] = j + i < cols ? (unsigned long long)__double_as_longlong(xr[j + i])
+                                        : 0ull;
+            }
+        };
+        int emax = 0;
+        bool any = false;
+        for (int j = threadIdx.x * 4; j < cols; j += Z_SLICE_THREADS * 4) {
+            unsigned long long b[4];
+            load4(j, b);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                emax = max(emax, (int)(b[i] >> 52) & 0x7ff);
+                any |= (b[i] << 1) != 0ull;
+            }
+        }
+        // a row of subnormal numbers counts as exponent 1, an all-zero row as none
+        emax = any ? max(emax, 1) : 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+        if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = emax;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < Z_SLICE_THREADS / 32; ++w) emax = max(emax, wmax[w]);
+        __syncthreads();
+        if (threadIdx.x == 0) out.e[r] = emax ? emax - 1022 : 0;
         const size_t off = (size_t)r * out.ld;
-        for (int j = lane; j < out.ld; j += 32) {
-            int dg[Z_ND];
+        for (int j = threadIdx.x * 4; j < ncol; j += Z_SLICE_THREADS * 4) {
+            unsigned long long b[4];
+            load4(j, b);
+            uint32_t dg[Z_ND][2];
 #pragma unroll
-            for (int d = 0; d < Z_ND; ++d) dg[d] = 0;
-            if (j < cols && mx > 0.0) {
-                // T = round(x 2^(55 - e)), |T| <= 2^55; digits by round-to-nearest
-                long long T = __double2ll_rn(ldexp(xr[j], BITS - e));
+            for (int i = 0; i < 4; ++i) {
+                long long T = emax ? oz64_fixed(b[i], emax) : 0ll;
 #pragma unroll
-                for (int d = 0; d < Z_ND - 1; ++d) {
+                for (int d = 0; d < Z_ND; ++d) {
                     const int sh = 8 * (Z_ND - 1 - d);
-                    const long long a = (T + (1ll << (sh - 1))) >> sh;
-                    dg[d] = (int)a;
-                    T -= a << sh;
+                    int v;
+                    if (d < Z_ND - 1) {
+                        const long long a = (T + (1ll << (sh - 1))) >> sh;
+                        v = (int)a;
+                        T -= a << sh;
+                    } else {
+                        v = (int)T;
+                    }
+                    // |v| <= 128: the upper half of its FP32 form is its BF16 form, exactly
+                    const uint32_t h = __float_as_uint((float)v) >> 16;
+                    if ((i & 1) == 0)
+                        dg[d][i >> 1] = h;
+                    else
+                        dg[d][i >> 1] |= h << 16;
                 }
-                dg[Z_ND - 1] = (int)T;
             }
 #pragma unroll
             for (int d = 0; d < Z_ND; ++d)
-                ((__nv_bfloat16*)out.s[d])[off + j] = __float2bfloat16_rn((float)dg[d]);
+                *(uint2*)((__nv_bfloat16*)out.s[d] + off + j) = make_uint2(dg[d][0], dg[d][1]);
         }
     }
 }
@@ -572,10 +703,8 @@ cdmpt_status oz64_slice(const double* x, int rows, int cols, int ld, const Oz64O
             set_error("FP64 Ozaki slicing: digit arrays missing");
             return CDMPT_ERR_ARG;
         }
-    const int wpb = 8;
-    int grid = (rows + wpb - 1) / wpb;
-    if (grid > 152 * 16) grid = 152 * 16;
-    k_oz64_slice<<<grid, 32 * wpb, 0, s>>>(x, rows, cols, ld, out, skip);
+    const int grid = rows < 152 * 16 ? rows : 152 * 16;
+    k_oz64_slice<<<grid, Z_SLICE_THREADS, 0, s>>>(x, rows, cols, ld, out, skip);
     count_launch();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -647,9 +776,22 @@ cdmpt_status gemm_oz64(int M, int N, int K, const Oz64Operand& X, const Oz64Oper
     p.lde = ep.lde;
     p.Dhi = nullptr;
     p.Dlo = nullptr;
-    p.sym = 0;   // full tiles: every element computed
+    p.sym = (ep.sym && M == N && p.trans_block == 0) ? 1 : 0;
     const int num_mt = (M + 2 * BM - 1) / (2 * BM);
-    const int tiles = num_mt * ((N + Z_BN - 1) / Z_BN);
+    const int num_nt = (N + Z_BN - 1) / Z_BN;
+    int tiles = num_mt * num_nt;
+    if (p.sym) {
+        tiles = 0;
+        for (int j = 0; j < num_nt; ++j) tiles += j / 4 + 1;
+    }
+    // a power of two alpha goes into the exponent of the rounded sum (neg < 0: alpha is none)
+    int alpha_exp = 0, alpha_neg = -1;
+    if (std::fabs(std::frexp(ep.alpha, &alpha_exp)) == 0.5 && alpha_exp > -900 && alpha_exp < 900) {
+        alpha_exp -= 1;
+        alpha_neg = ep.alpha < 0.0 ? 1 : 0;
+    } else {
+        alpha_exp = 0;
+    }
     const int clusters = tiles < max_clusters ? tiles : max_clusters;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * clusters);
@@ -664,7 +806,7 @@ cdmpt_status gemm_oz64(int M, int N, int K, const Oz64Operand& X, const Oz64Oper
     cfg.attrs = &a;
     cfg.numAttrs = 1;
     cudaError_t e = cudaLaunchKernelEx(&cfg, kern, maps, p, (const int*)X.e, (const int*)Y.e, K,
-                                       num_mt, tiles, skip, device_error_word());
+                                       num_mt, tiles, alpha_exp, alpha_neg, skip, device_error_word());
     count_launch();
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {

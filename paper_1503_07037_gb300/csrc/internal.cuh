@@ -258,13 +258,13 @@ struct Oz64Operand {
     int* e = nullptr;
     int ld = 0;
 };
-// One warp per row: digits of x (rows x cols, leading dimension ld) into out (out.ld >= cols,
+// One block per row: digits of x (rows x cols, leading dimension ld) into out (out.ld >= cols,
 // zeros in the padding). Does nothing while *skip != 0 (skip may be null).
 cdmpt_status oz64_slice(const double* x, int rows, int cols, int ld, const Oz64Operand& out,
                         const double* skip, cudaStream_t s);
 // D = alpha X Y^T + beta C + gamma I_blocks in FP64 from the digits of X (M x K) and Y (N x K),
-// K <= 16384; full tiles (ep.sym is ignored), transposed placement and fused dot as the other
-// engines. Does nothing while *skip != 0.
+// K <= 16384; transposed placement, fused dot and ep.sym (upper-triangle tiles, mirrored) as the
+// other engines. Does nothing while *skip != 0.
 cdmpt_status gemm_oz64(int M, int N, int K, const Oz64Operand& X, const Oz64Operand& Y,
                        double* D, int ldd, const Epilogue<double>& ep, const double* skip,
                        cudaStream_t s);
