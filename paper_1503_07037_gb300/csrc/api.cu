@@ -1154,7 +1154,7 @@ cdmpt_status cdmpt_gemm_f64(int M, int Ncols, int K, const double* X, int ldx, c
     ep.gamma = gamma;
     ep.diag_block = diag_block;
     ep.trans_block = trans_block > 0 ? trans_block : 0;
-    ep.sym = trans_block < 0;
+    ep.sym = false;   // every element is computed
     ep.dot = dot;
     ep.E = E;
     ep.lde = lde;

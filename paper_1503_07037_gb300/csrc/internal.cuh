@@ -91,6 +91,8 @@ cdmpt_status check_device_error(cudaStream_t s);
 template <typename T>
 cdmpt_status gemm_simt(int M, int N, int K, const T* X, int ldx, const T* Y, int ldy, T* D,
                        int ldd, const Epilogue<T>& ep, const double* skip, cudaStream_t s);
+// Whether an M x N x K FP64 product is short enough for the DFMA tiles of gemm_simt
+bool small_f64(int M, int N, int K, bool sym);
 
 // Block-norm screening of one tcgen05 product X Y^T (M x N, depth K): the bit mask of
 // the k-slices each 128 x 128 output tile computes (see GemmProblem), nmw words per

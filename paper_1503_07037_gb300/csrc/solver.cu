@@ -353,10 +353,15 @@ template <typename T>
 cdmpt_status Solver<T>::gemm(Context& cx, int M, int Nc, int K, const Operand<T>& X,
                              const Operand<T>& Y, T* D, const Epilogue<T>& ep, const double* skip,
                              int engine_override) {
-    const int engine = engine_of(cx, engine_override);
+    int engine = engine_of(cx, engine_override);
+    if constexpr (sizeof(T) == 8) {
+        // short FP64 products: DFMA tiles beat slicing plus the digit kernel's latency
+        if (engine == CDMPT_GEMM_TC_OZAKI && small_f64(M, Nc, K, ep.sym && M == Nc))
+            engine = CDMPT_GEMM_SIMT;
+    }
     // flops the product needs: a symmetric result on the tensor-core engines is
     // computed on its upper-triangular tiles only, N (N + 1) K instead of 2 N^2 K
-    const bool sym_tc = ep.sym && M == Nc && engine != CDMPT_GEMM_SIMT;
+    const bool sym_tc = ep.sym && M == Nc && (engine != CDMPT_GEMM_SIMT || sizeof(T) == 8);
     const double flops = sym_tc ? (double)M * (M + 1) * K : 2.0 * M * (double)Nc * K;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (cx.profile) {
@@ -990,7 +995,7 @@ cdmpt_status Solver<T>::step0(Context& cx, int k, int engine, double tol, int ma
             CDMPT_TRY(poly_eval(cx, W_[k], p, 1.0, engine, &E));
         }
         CDMPT_TRY(gemm(cx, N_, N_, N_, Z_[k].op(), E->op(), Z_[k + 1].x, ep, nullptr, engine));
-        if (engine == CDMPT_GEMM_SIMT)   // full tiles, not mirrored
+        if (engine_of(cx, engine) == CDMPT_GEMM_SIMT)   // full tiles, not mirrored
             CDMPT_TRY(Ew<T>::symmetrize(Z_[k + 1].x, N_, ld, 1, cx.stream, Z_[k + 1].hi,
                                         Z_[k + 1].lo));
         *iters += p.degree();
