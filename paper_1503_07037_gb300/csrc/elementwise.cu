@@ -214,6 +214,11 @@ __global__ void k_cg_scalar_init(double* sc, double tol2, double tol2_r0, const 
     sc[CG_DONE] = (sc[CG_RR] <= thresh) ? 1.0 : 0.0;
 }
 
+__global__ void k_refine_ratio(double* v) {
+    if (v[1] > 0.0) v[2] = fmax(v[2], sqrt(v[0] / (4.0 * v[1])));
+    v[0] = v[1] = 0.0;
+}
+
 template <typename T>
 __global__ void k_dot(const T* __restrict__ A, const T* __restrict__ B, size_t nvec,
                       double* __restrict__ out, const double* __restrict__ skip) {
@@ -827,6 +832,12 @@ cdmpt_status split_tf32(const float* X, size_t count, float* hi, float* lo, cuda
 
 template struct Ew<float>;
 template struct Ew<double>;
+
+cdmpt_status refine_ratio(double* v, cudaStream_t s) {
+    k_refine_ratio<<<1, 1, 0, s>>>(v);
+    LAUNCH_CHECK();
+    return CDMPT_OK;
+}
 
 cdmpt_status cg_scalar_step(double* sc, cudaStream_t s) {
     k_cg_scalar_step<<<1, 1, 0, s>>>(sc);

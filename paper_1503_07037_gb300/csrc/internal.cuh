@@ -291,6 +291,9 @@ cdmpt_status add(float* hi, float* lo, const float* d, size_t count, cudaStream_
                  float* thi = nullptr, float* tlo = nullptr);
 cdmpt_status symmetrize(float* hi, float* lo, int N, int ld, int blocks, cudaStream_t s,
                         float* thi = nullptr, float* tlo = nullptr);
+// (hi, lo) += (d + d^T) / 2 for one N x N matrix (a symmetric pair stays exactly symmetric)
+cdmpt_status add_sym(float* hi, float* lo, const float* d, int N, int ld, cudaStream_t s,
+                     float* thi = nullptr, float* tlo = nullptr);
 cdmpt_status add_diag(float* hi, float* lo, int N, int ld, int blocks, double shift,
                       cudaStream_t s, float* thi = nullptr, float* tlo = nullptr);
 // out = a (hi + lo) + b_diag I in FP64
@@ -305,6 +308,8 @@ cdmpt_status cg_scalar_step(double* sc, cudaStream_t s);
 // tol2_ref *ref) (ref: a device scalar, or null).
 cdmpt_status cg_scalar_init(double* sc, double tol2, double tol2_r0, cudaStream_t s,
                             const double* ref = nullptr, double tol2_ref = 0.0);
+// v = [||r||^2, ||z||^2, worst]: worst = max(worst, ||r|| / (2 ||z||)), the first two back to zero
+cdmpt_status refine_ratio(double* v, cudaStream_t s);
 cdmpt_status gershgorin(const double* H, int N, int ld, double* out2, cudaStream_t s);
 cdmpt_status gershgorin_noalloc(const double* H, int N, int ld, double* out2, cudaStream_t s);
 // Count of kernel launches issued by this thread (for statistics).

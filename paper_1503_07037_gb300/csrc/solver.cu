@@ -59,6 +59,9 @@ enum Slot {
     S_ZZ = 9,       // ||Z_n||_F^2
     S_TRQ = 10,     // Tr Q
     S_REF = 11,     // ||ref||_F^2 of the running CG solve's absolute tolerance
+    S_RR = 12,      // ||r||_F^2 and ||Z_k||_F^2 of the running refinement step, and the largest
+    S_RZ = 13,      // ||r|| / ||2 Z_k|| of the pass so far
+    S_WORST = 14,
     S_TRZ1 = 16,    // Tr Z1_d (d < 16)
     S_ALPHA = 32,   // sum P1_d * H1_d (d < 16)
     S_FE = 48,      // free energy and Omega terms: traces and dots (5 slots)
@@ -1094,8 +1097,7 @@ template <typename T>
 cdmpt_status Solver<T>::correct(Context& cx, int k, const T* d) {
     if constexpr (sizeof(T) == 4) {
         if (Z_[k].xl) {
-            CDMPT_TRY(pair::add(Z_[k].x, Z_[k].xl, d, blk_, cx.stream));
-            return pair::symmetrize(Z_[k].x, Z_[k].xl, N_, ld, 1, cx.stream, Z_[k].hi, Z_[k].lo);
+            return pair::add_sym(Z_[k].x, Z_[k].xl, d, N_, ld, cx.stream, Z_[k].hi, Z_[k].lo);
         }
     }
     CDMPT_TRY(Ew<T>::axpby(Z_[k].x, d, blk_, 1.0, 1.0, nullptr, cx.stream));
@@ -1116,9 +1118,13 @@ cdmpt_status Solver<T>::refine(Context& cx, const cdmpt_opts& o, int n, int k_hp
                                double* max_rel_res) {
     int total = 0;
     double worst = 0.0;
+    // a BF16 sweep's Z_{k+1} (1e-2) gives too coarse an inverse for the first pass
+    const bool closed = closed_tangent(o) &&
+                        !(o.precision == CDMPT_MIXED_BF16 && cx.st->refine_passes == 0);
+    if (closed) CDMPT_CUDA_TRY(cudaMemsetAsync(sc_ + S_RR, 0, 3 * sizeof(double), cx.stream));
     for (int k = 0; k < n; ++k) {
         if (k >= k_hp) {
-            CDMPT_TRY(residual_hp(cx, k));
+            CDMPT_TRY(residual_hp(cx, k, closed ? sc_ + S_RR : nullptr));
         } else {
             {   // W_k from the refined Z_k
                 Epilogue<T> ep;
@@ -1148,9 +1154,39 @@ cdmpt_status Solver<T>::refine(Context& cx, const cdmpt_opts& o, int n, int k_hp
                 ep.beta = 1.0;
                 ep.C = S_.x;
                 ep.ldc = ld;
+                if (closed) {
+                    ep.Dhi = RHS_.hi;
+                    ep.Dlo = RHS_.lo;
+                    ep.dot = sc_ + S_RR;
+                }
                 CDMPT_TRY(gemm(cx, N_, N_, N_, Z_[k + 1].op(), W_[k].op(), RHS_.x, ep, nullptr,
                                CDMPT_GEMM_TC_3XTF32));
             }
+        }
+        if (closed) {
+            // correction d = r A_k^-1 with A_k^-1 = I - 1/2 Z_{k+1} Z_k (tangent_step) of the stored
+            // trajectory, good to the 1e-4 of its Z_{k+1}: two one-pass TF32 products, one of them
+            // on half the tiles, gain the three digits that took CG two to three whole ones, its
+            // vector passes and a host read-back per step
+            Epilogue<T> eb;
+            eb.Dhi = A1_.hi;
+            eb.Dlo = A1_.lo;
+            eb.sym = true;
+            CDMPT_TRY(gemm(cx, N_, N_, N_, Z_[k + 1].op(), Z_[k].op(), A1_.x, eb, nullptr,
+                           CDMPT_GEMM_TC_TF32));
+            Epilogue<T> ed;
+            ed.alpha = -0.5;
+            ed.beta = 1.0;
+            ed.C = RHS_.x;
+            ed.ldc = ld;
+            CDMPT_TRY(gemm(cx, N_, N_, N_, RHS_.op(), A1_.op(), P_.x, ed, nullptr,
+                           CDMPT_GEMM_TC_TF32));
+            total += 1;
+            // ||Z_k||^2 = Tr W_k; the pass's worst ratio stays on the device until its end
+            CDMPT_TRY(Ew<T>::trace(W_[k].x, N_, ld, 1, sc_ + S_RZ, cx.stream));
+            CDMPT_TRY(refine_ratio(sc_ + S_RR, cx.stream));
+            CDMPT_TRY(correct(cx, k + 1, P_.x));
+            continue;
         }
         // correction d (I + W_k) = r with one-pass TF32 iterations
         CgArgs a;
@@ -1172,6 +1208,10 @@ cdmpt_status Solver<T>::refine(Context& cx, const cdmpt_opts& o, int n, int k_hp
         const double zz = cx.pinned[S_ZZ];
         if (zz > 0) worst = std::max(worst, std::sqrt(bb / (4.0 * zz)));
         CDMPT_TRY(correct(cx, k + 1, A1_.x));
+    }
+    if (closed) {
+        CDMPT_TRY(read_scalars(cx, sc_, S_NSLOTS));
+        worst = cx.pinned[S_WORST];
     }
     *cg_iters = total;
     *max_rel_res = worst;
@@ -1241,7 +1281,7 @@ cdmpt_status Solver<T>::gemm_hp(Context& cx, const OzOperand& X, const OzOperand
 // of the pair-stored trajectory: the FP32 part and TF32 split of W_k replace the stored W_k, its
 // low part goes to wl_, and the linear part of r is formed in double-float in the epilogue.
 template <typename T>
-cdmpt_status Solver<T>::residual_hp(Context& cx, int k) {
+cdmpt_status Solver<T>::residual_hp(Context& cx, int k, double* rr) {
     if constexpr (sizeof(T) != 4) {
         set_error("FP64-class residuals need the pair-stored FP32 trajectory");
         return CDMPT_ERR_UNSUPPORTED;
@@ -1265,6 +1305,11 @@ cdmpt_status Solver<T>::residual_hp(Context& cx, int k) {
         CDMPT_TRY(oz_slice(Z_[k + 1].x, Z_[k + 1].xl, N_, N_, ld, oz_[2], cx.stream));
         OzEpi ep;
         ep.D = RHS_.x;
+        if (rr) {
+            ep.Dthi = RHS_.hi;
+            ep.Dtlo = RHS_.lo;
+            ep.dot = rr;
+        }
         ep.ldd = ld;
         ep.alpha = -1.f;
         ep.b1 = 2.f;

@@ -215,8 +215,9 @@ private:
     cdmpt_status refine(Context& cx, const cdmpt_opts& o, int n, int k_hp, int* cg_iters,
                         double* max_rel_res);
     // W_k and the residual of step k (into RHS_) from Ozaki-sliced products of the
-    // pair-stored trajectory (FP64-class residuals).
-    cdmpt_status residual_hp(Context& cx, int k);
+    // pair-stored trajectory (FP64-class residuals); rr (device, or null) receives += ||r||^2
+    // and the residual its TF32 split.
+    cdmpt_status residual_hp(Context& cx, int k, double* rr);
     // D = op(X Y^T) by gemm_oz, with the profile events and statistics of gemm()
     cdmpt_status gemm_hp(Context& cx, const OzOperand& X, const OzOperand& Y, const OzEpi& ep,
                          int nd = kOzDigits);
