@@ -754,14 +754,170 @@ cdmpt_status init_z0_batch(cdmpt_batch* b, const std::vector<const double*>& ski
     return run_ew(b, G_PAIR_INIT, dp);
 }
 
+// One step Z_{k+1} = 2 Z_k p(W_k) of every unconverged system by matrix polynomials (as
+// Solver::step0 and poly_eval, one grouped launch per product). All systems take the shape that
+// the one with the largest spectral bound needs, each with its own coefficients. *done = false
+// if that exceeds max_degree (the caller then solves by CG).
+cdmpt_status poly_step_batch(cdmpt_batch* b, int k, const std::vector<double>& zb, int engine,
+                             double tol, int max_degree, int* degree, bool* done) {
+    const int G = b->B;
+    std::vector<InversePoly> pl(G);
+    *done = false;
+    int s = 0, r = 0, deg = 0;
+    for (int i = 0; i < G; ++i) {
+        if (b->sys[i].converged) continue;
+        InversePoly& q = pl[i];
+        if (!q.fit(1.0, 0.0, zb[i] * zb[i], 0.5 * tol, max_degree)) return CDMPT_OK;
+        if (q.degree() > deg) {
+            deg = q.degree();
+            s = q.s;
+            r = q.r;
+        }
+    }
+    if (deg == 0 || s > 4) return CDMPT_OK;
+    for (int i = 0; i < G; ++i)
+        if (!b->sys[i].converged &&
+            !pl[i].fit(1.0, 0.0, zb[i] * zb[i], 0.5 * tol, std::max(max_degree, deg), s, r))
+            return CDMPT_OK;
+    // one grouped symmetric product; spec(sy, q, g) fills X, Y and the epilogue per system
+    auto product = [&](auto spec) -> cdmpt_status {
+        std::vector<GemmSpec> g;
+        for (int i = 0; i < G; ++i) {
+            Sys& sy = b->sys[i];
+            if (sy.converged) continue;
+            GemmSpec e;
+            e.rows = sy.N;
+            e.skip = nullptr;
+            spec(sy, pl[i], e);
+            e.p.sym = 1;
+            g.push_back(e);
+            add_flops(b, sym_flops(b, sy.N), engine);
+        }
+        return grouped_gemm(b, g, engine);
+    };
+    auto to = [](const Sys& sy, const Mat& D, double alpha, double beta, const float* C,
+                 double gamma, bool split) {
+        EpiParams<float> p = epi(D.x, sy.N, sy.N, sy.ld, (float)alpha, (float)beta, C, (float)gamma);
+        if (split) {
+            p.Dhi = D.hi;
+            p.Dlo = D.lo;
+        }
+        return p;
+    };
+    using MatOf = Mat Sys::*;
+    MatOf E = nullptr;
+    if (s == 2 && r == 0) {
+        CDMPT_TRY(product([&](Sys& sy, const InversePoly& q, GemmSpec& e) {
+            e.X = e.Y = &sy.W[k];
+            e.p = to(sy, sy.A1, q.a[2], q.a[1] - 2.0 * q.c * q.a[2], sy.W[k].x,
+                     (q.a[0] - 1.0) - q.a[1] * q.c + q.a[2] * q.c * q.c, true);
+        }));
+        E = &Sys::A1;
+    } else if (s > 1) {
+        // powers S^2 (A1), S^3 (RHS, or R below S^4), S^4 (RHS)
+        MatOf pw[4] = {nullptr, &Sys::A1, s == 3 ? &Sys::RHS : &Sys::R, &Sys::RHS};
+        CDMPT_TRY(product([&](Sys& sy, const InversePoly& q, GemmSpec& e) {
+            e.X = e.Y = &sy.W[k];
+            e.p = to(sy, sy.A1, 1.0, -2.0 * q.c, sy.W[k].x, q.c * q.c, true);
+        }));
+        if (s >= 3)
+            CDMPT_TRY(product([&](Sys& sy, const InversePoly& q, GemmSpec& e) {
+                e.X = &sy.A1;
+                e.Y = &sy.W[k];
+                e.p = to(sy, sy.*pw[2], 1.0, -q.c, sy.A1.x, 0.0, s == 3);
+            }));
+        if (s == 4)
+            CDMPT_TRY(product([&](Sys& sy, const InversePoly&, GemmSpec& e) {
+                e.X = e.Y = &sy.A1;
+                e.p = to(sy, sy.RHS, 1.0, 0.0, nullptr, 0.0, true);
+            }));
+        // coefficient blocks: the lower ones in plain buffers (s > 2), the top one in P
+        MatOf low[3] = {s == 3 ? &Sys::R : &Sys::Q, s == 3 ? &Sys::Q : &Sys::S,
+                        s == 3 ? &Sys::S : &Sys::R};
+        std::vector<GrpPoly> d;
+        long long maxc = 0;
+        const int nb = s > 2 ? r + 1 : 1;
+        for (int i = 0; i < G; ++i) {
+            Sys& sy = b->sys[i];
+            if (sy.converged) continue;
+            const InversePoly& q = pl[i];
+            GrpPoly e;
+            std::memset(&e, 0, sizeof(e));
+            e.P[0] = sy.W[k].x;
+            for (int j = 1; j < s; ++j) e.P[j] = (sy.*pw[j]).x;
+            for (int t = 0; t + 1 < nb; ++t) {
+                e.out[t] = (sy.*low[t]).x;
+                for (int j = 0; j < s; ++j) e.coef[t][j] = (float)q.a[t * s + j];
+            }
+            if (nb > 1) e.coef[0][0] = (float)(q.a[0] - 1.0);
+            e.out[nb - 1] = sy.P.x;
+            for (int j = 0; j <= s; ++j) e.coef[nb - 1][j] = (float)q.a[r * s + j];
+            e.hi = sy.P.hi;
+            e.lo = sy.P.lo;
+            e.c = (float)q.c;
+            e.count = (long long)sy.blk;
+            e.ld = sy.ld;
+            maxc = std::max(maxc, e.count);
+            d.push_back(e);
+        }
+        const GrpPoly* dev = nullptr;
+        CDMPT_TRY(stage(b, d, &dev));
+        CDMPT_TRY(grouped_poly(dev, (int)d.size(), s, nb, maxc, b->cx.stream));
+        MatOf H = &Sys::P, Hn = s == 2 ? &Sys::RHS : &Sys::A1;
+        for (int t = r - 1; t >= 0; --t) {
+            CDMPT_TRY(product([&](Sys& sy, const InversePoly& q, GemmSpec& e) {
+                e.X = &(sy.*H);
+                e.Y = &(sy.*pw[s - 1]);
+                if (s == 2) {
+                    const double a1 = q.a[2 * t + 1];
+                    e.p = to(sy, sy.*Hn, 1.0, a1, sy.W[k].x,
+                             q.a[2 * t] - (t == 0 ? 1.0 : 0.0) - a1 * q.c, true);
+                } else {
+                    e.p = to(sy, sy.*Hn, 1.0, 1.0, (sy.*low[t]).x, 0.0, true);
+                }
+            }));
+            std::swap(H, Hn);
+        }
+        E = H;
+    }
+    CDMPT_TRY(product([&](Sys& sy, const InversePoly& q, GemmSpec& e) {   // Z_{k+1}
+        const double h = 2.0 * q.c;
+        e.X = &sy.Z[k];
+        e.Y = E ? &(sy.*E) : &sy.W[k];
+        e.p = to(sy, sy.Z[k + 1], E ? 2.0 : -2.0 * (1.0 - 0.8284 * h), 2.0, sy.Z[k].x, 0.0, true);
+    }));
+    if (b->tile_bn == 64) {   // 64-column tiles compute symmetric results whole
+        std::vector<GrpEw> dsym;
+        for (int i = 0; i < G; ++i) {
+            Sys& sy = b->sys[i];
+            if (sy.converged) continue;
+            GrpEw y = ewd(sy.Z[k + 1].x, nullptr, sy.Z[k + 1].hi, sy.Z[k + 1].lo);
+            y.rows = sy.N; y.ld = sy.ld; y.N = sy.N;
+            dsym.push_back(y);
+        }
+        CDMPT_TRY(run_tiles(b, dsym, 1, grouped_symmetrize));
+    }
+    *degree = deg;
+    *done = true;
+    return CDMPT_OK;
+}
+
 // One 0th-order pass for the systems whose inactive flag is 0, with products on
-// engine and CG to relative residual tol.
+// engine, by matrix polynomials (or CG to relative residual tol where the iteration cap is
+// below their degree).
 cdmpt_status sweep_batch(cdmpt_batch* b, int n, int* iters_out, int engine, double tol) {
     const int G = b->B;
     std::vector<const double*> skip(G);
     for (int i = 0; i < G; ++i) skip[i] = b->inactive + i;
     CDMPT_TRY(init_z0_batch(b, skip));
     int total = 0, hint = 1;
+    // |Z_k| <= tanh(2^k atanh |Z_0|), with a margin for the rounding of the products
+    std::vector<double> zb(G);
+    const double margin = engine == CDMPT_GEMM_TC_TF32 ? 1e-3 : 1e-6;
+    for (int i = 0; i < G; ++i) {
+        const Sys& sy = b->sys[i];
+        zb[i] = std::min(sy.s2 * std::max(sy.gmax - sy.mu, sy.mu - sy.gmin) * (1.0 + margin), 1.0);
+    }
     for (int k = 0; k < n; ++k) {
         std::vector<GemmSpec> gw, gr;
         std::vector<BCg> cg(G);
@@ -808,10 +964,21 @@ cdmpt_status sweep_batch(cdmpt_batch* b, int n, int* iters_out, int engine, doub
         }
         if (b->tile_bn == 0) CDMPT_TRY(tune_tiles(b, gw));   // first product of the batch
         CDMPT_TRY(grouped_gemm(b, gw, engine));
+        for (int i = 0; i < G; ++i)
+            if (!b->sys[i].converged) add_flops(b, sym_flops(b, b->sys[i].N), engine);
+        int it = 0;
+        bool done = false;
+        CDMPT_TRY(poly_step_batch(b, k, zb, engine, tol, std::min(b->opts.cg_maxit, 16), &it,
+                                  &done));
+        for (double& z : zb) z = std::min(2.0 * z / (1.0 + z * z) * (1.0 + margin), 1.0);
+        if (done) {
+            total += it;
+            CDMPT_TRY(run_ew(b, G_ZERO, dzl));
+            continue;
+        }
         CDMPT_TRY(grouped_gemm(b, gr, engine));
         for (int i = 0; i < G; ++i)
-            if (!b->sys[i].converged) add_flops(b, 2.0 * sym_flops(b, b->sys[i].N), engine);
-        int it = 0;
+            if (!b->sys[i].converged) add_flops(b, sym_flops(b, b->sys[i].N), engine);
         // mirrored CG products only in the one-pass sweeps of mixed precision (refined later);
         // the accurate sweeps (tol <= 1e-6) also stop relative to the new iterate
         CDMPT_TRY(cg_batch(b, cg, 1.0, 1.0, tol, skip, hint, &it, engine != kEngine, engine, -1,
@@ -837,18 +1004,13 @@ cdmpt_status hp_join_lanes(cdmpt_batch* b) {
     return CDMPT_OK;
 }
 
-// W_k and the residual 2 Z_k - Z_{k+1} - Z_{k+1} W_k of step k from Ozaki-sliced products of
-// the pair-stored trajectory, for every active system one after another (they share the
-// digit buffers); W_k's FP32 part and split replace the stored W_k, the residual goes to RHS.
-// The work goes to side lanes forked from the batch's stream; join: the batch's stream waits
-// for them before returning (else hp_join_lanes does, after more work on the batch's stream).
-cdmpt_status residual_batch_hp(cdmpt_batch* b, int k, const std::vector<char>& active,
-                               bool join = true) {
+// Forks *lanes side lanes (one per active system, at most hp_nlanes) from the batch's stream.
+cdmpt_status hp_fork_lanes(cdmpt_batch* b, const std::vector<char>& active, int* lanes) {
     cudaStream_t s = b->cx.stream;
     int nact = 0;
     for (int i = 0; i < b->B; ++i) nact += active[i] ? 1 : 0;
-    if (nact == 0) return CDMPT_OK;
-    const int L = std::min(nact, b->hp_nlanes);
+    const int L = *lanes = std::min(nact, b->hp_nlanes);
+    if (L == 0) return CDMPT_OK;
     if (!b->hp_fork) {
         CDMPT_CUDA_TRY(cudaEventCreateWithFlags(&b->hp_fork, cudaEventDisableTiming));
         for (int l = 0; l < cdmpt_batch::kHpLanes; ++l) {
@@ -859,6 +1021,53 @@ cdmpt_status residual_batch_hp(cdmpt_batch* b, int k, const std::vector<char>& a
     // the lanes start after everything queued on the batch's stream
     CDMPT_CUDA_TRY(cudaEventRecord(b->hp_fork, s));
     for (int l = 0; l < L; ++l) CDMPT_CUDA_TRY(cudaStreamWaitEvent(b->hp_st[l], b->hp_fork, 0));
+    return CDMPT_OK;
+}
+
+// B_k = Z_{k+1} Z_k (sy.S.x) from four Ozaki digits of the pair-stored trajectory for the flagged
+// systems (see Solver::step_product), on side lanes.
+cdmpt_status step_product_hp(cdmpt_batch* b, int k, const std::vector<char>& active) {
+    int L = 0;
+    CDMPT_TRY(hp_fork_lanes(b, active, &L));
+    constexpr int nd = 4;
+    int j = 0;
+    for (int i = 0; i < b->B; ++i) {
+        if (!active[i]) continue;
+        const int l = j++ % L;
+        cudaStream_t ls = b->hp_st[l];
+        OzOperand* oz = b->oz[l];
+        Sys& sy = b->sys[i];
+        for (int a = 0; a < 2; ++a) {
+            oz[a].ld = sy.ld;
+            CDMPT_TRY(oz_slice(sy.Z[k + a].x, sy.Z[k + a].xl, sy.N, sy.N, sy.ld, oz[a], ls, nd));
+        }
+        OzEpi e;
+        e.sym = 2;
+        e.D = sy.S.x;
+        e.ldd = sy.ld;
+        e.alpha = 1.f;
+        CDMPT_TRY(gemm_oz(sy.N, sy.N, sy.N, oz[1], oz[0], e, ls, nd));
+        if (b->cx.st) {
+            const double f = sym_flops(b, sy.N);
+            b->cx.st->gemm_launches += 1;
+            b->cx.st->gemm_flops += f;
+            b->cx.st->tensor_flops += oz_products(nd) * f;
+        }
+    }
+    b->hp_lanes = L;
+    return CDMPT_OK;
+}
+
+// W_k and the residual 2 Z_k - Z_{k+1} - Z_{k+1} W_k of step k from Ozaki-sliced products of
+// the pair-stored trajectory, for every active system one after another (they share the
+// digit buffers); W_k's FP32 part and split replace the stored W_k, the residual goes to RHS.
+// The work goes to side lanes forked from the batch's stream; join: the batch's stream waits
+// for them before returning (else hp_join_lanes does, after more work on the batch's stream).
+cdmpt_status residual_batch_hp(cdmpt_batch* b, int k, const std::vector<char>& active,
+                               bool join = true) {
+    int L = 0;
+    CDMPT_TRY(hp_fork_lanes(b, active, &L));
+    if (L == 0) return CDMPT_OK;
     int j = 0;
     for (int i = 0; i < b->B; ++i) {
         if (!active[i]) continue;
@@ -881,6 +1090,8 @@ cdmpt_status residual_batch_hp(cdmpt_batch* b, int k, const std::vector<char>& a
         CDMPT_TRY(oz_slice(sy.Z[k + 1].x, sy.Z[k + 1].xl, sy.N, sy.N, sy.ld, oz[2], ls));
         OzEpi r;
         r.D = sy.RHS.x;
+        r.Dthi = sy.RHS.hi;
+        r.Dtlo = sy.RHS.lo;
         r.ldd = sy.ld;
         r.alpha = -1.f;
         r.b1 = 2.f;
@@ -904,9 +1115,10 @@ cdmpt_status residual_batch_hp(cdmpt_batch* b, int k, const std::vector<char>& a
 
 // One refinement pass of the stored trajectories (mixed precision), for the systems whose
 // inactive flag is 0 (active[i] on the host): per step, W_k = Z_k Z_k and the residual
-// 2 Z_k - Z_{k+1} - Z_{k+1} W_k, then the correction d (I + W_k) = residual by CG with
-// one-pass TF32 products (relative residual 1e-3), Z_{k+1} += d added to the pair,
-// symmetrised. A system's steps form W_k and the residual with grouped split-TF32 products
+// 2 Z_k - Z_{k+1} - Z_{k+1} W_k, then the correction d = residual (I + W_k)^-1 with
+// one-pass TF32 products (the inverse I - 1/2 Z_{k+1} Z_k of the stored trajectory, as in
+// Solver::refine; CG to a relative residual of 1e-3 where the caller caps its iterations
+// low), Z_{k+1} += d added to the pair, symmetrised. A system's steps form W_k and the residual with grouped split-TF32 products
 // (full tiles for the residual: the stored Z_{k+1} does not commute with W_k to first order
 // in its error), except, once the system is in its FP64-class passes (Sys::hp), the steps
 // k >= Sys::khp, which use Ozaki-sliced products.
@@ -915,6 +1127,7 @@ cdmpt_status refine_batch(cdmpt_batch* b, int n, const std::vector<char>& active
     const int G = b->B;
     std::vector<const double*> skip(G);
     for (int i = 0; i < G; ++i) skip[i] = b->inactive + i;
+    const bool closed = krylov_degree(b->opts.cg_tol) <= b->opts.cg_maxit;
     int total = 0;
     for (int k = 0; k < n; ++k) {
         std::vector<GemmSpec> gw, gr;
@@ -964,6 +1177,10 @@ cdmpt_status refine_batch(cdmpt_batch* b, int n, const std::vector<char>& active
             r.rows = sy.N;
             r.Y = &sy.W[k];
             r.p = epi(sy.RHS.x, sy.N, sy.N, sy.ld, -1.f, 1.f, sy.S.x);
+            if (closed) {
+                r.p.Dhi = sy.RHS.hi;
+                r.p.Dlo = sy.RHS.lo;
+            }
             r.skip = skip[i];
             gr.push_back(r);
         }
@@ -979,6 +1196,43 @@ cdmpt_status refine_batch(cdmpt_batch* b, int n, const std::vector<char>& active
                 const double nn = b->sys[i].N;
                 add_flops(b, sym_flops(b, b->sys[i].N) + 2.0 * nn * nn * nn);
             }
+        }
+        if (closed) {
+            std::vector<GemmSpec> gb, gd;
+            std::vector<GrpEw> dc;
+            for (int i = 0; i < G; ++i) {
+                if (!active[i]) continue;
+                Sys& sy = b->sys[i];
+                GemmSpec e;                  // B = Z_{k+1} Z_k
+                e.X = &sy.Z[k + 1];
+                e.rows = sy.N;
+                e.Y = &sy.Z[k];
+                e.p = epi(sy.A1.x, sy.N, sy.N, sy.ld);
+                e.p.sym = 1;
+                e.p.Dhi = sy.A1.hi;
+                e.p.Dlo = sy.A1.lo;
+                e.skip = nullptr;
+                gb.push_back(e);
+                GemmSpec f;                  // d = r - 1/2 r B
+                f.X = &sy.RHS;
+                f.rows = sy.N;
+                f.Y = &sy.A1;
+                f.p = epi(sy.P.x, sy.N, sy.N, sy.ld, -0.5f, 1.f, sy.RHS.x);
+                f.skip = nullptr;
+                gd.push_back(f);
+                GrpEw c = ewd(sy.Z[k + 1].x, sy.Z[k + 1].xl, sy.Z[k + 1].hi, sy.Z[k + 1].lo);
+                c.p4 = sy.P.x;
+                c.rows = sy.N; c.ld = sy.ld; c.N = sy.N;
+                dc.push_back(c);
+                const double nn = sy.N;
+                add_flops(b, sym_flops(b, sy.N) + 2.0 * nn * nn * nn, CDMPT_GEMM_TC_TF32);
+            }
+            CDMPT_TRY(grouped_gemm(b, gb, CDMPT_GEMM_TC_TF32));
+            CDMPT_TRY(hp_join_lanes(b));
+            CDMPT_TRY(grouped_gemm(b, gd, CDMPT_GEMM_TC_TF32));
+            CDMPT_TRY(run_tiles(b, dc, 1, grouped_pair_add_sym));
+            total += 1;
+            continue;
         }
         CDMPT_TRY(hp_join_lanes(b));
         int it = 0;
@@ -1029,7 +1283,7 @@ cdmpt_status alloc_batch(cdmpt_batch* b, int n) {
     double* scal = nullptr;
     CDMPT_TRY(grab(b, (size_t)B * kSlots * sizeof(double), (void**)&scal));
     CDMPT_TRY(grab(b, (size_t)B * sizeof(double), (void**)&b->inactive));
-    b->maps_cap = B * (8 * n + 16) * 4;
+    b->maps_cap = B * (16 * n + 32) * 4;
     CDMPT_TRY(grab(b, (size_t)b->maps_cap * sizeof(CUtensorMap), (void**)&b->maps_dev));
     CDMPT_TRY(grab(b, (size_t)B * sizeof(GemmProblem), (void**)&b->it_gemm));
     CDMPT_TRY(grab(b, (size_t)3 * B * sizeof(GrpEw), (void**)&b->it_ew));
@@ -1132,6 +1386,7 @@ cdmpt_status cdmpt_batch_create(const cdmpt_opts* opts, int B, const int* N, int
     b->slot_bytes = std::max<size_t>(64 * 1024, (size_t)B * 16 * sizeof(GrpEw));
     b->slot_bytes = std::max<size_t>(b->slot_bytes, (size_t)B * D * sizeof(GrpEw) + 1024);
     b->slot_bytes = std::max<size_t>(b->slot_bytes, (size_t)B * sizeof(GemmProblem) + 1024);
+    b->slot_bytes = std::max<size_t>(b->slot_bytes, (size_t)B * sizeof(GrpPoly) + 1024);
     b->stage_slots = 512;
     if (cudaMallocHost((void**)&b->stage_host, b->slot_bytes * b->stage_slots) != cudaSuccess ||
         cudaMalloc((void**)&b->stage_dev, b->slot_bytes * b->stage_slots) != cudaSuccess ||
@@ -1413,7 +1668,63 @@ cdmpt_status cdmpt_batch_solve(cdmpt_batch* b, const double* beta, const double*
         }
         CDMPT_TRY(run_ew(b, G_INIT_Z, d));
         int total = 0, hint = 1;
-        for (int k = 0; k < n; ++k) {
+        const bool closed = krylov_degree(b->opts.cg_tol) <= b->opts.cg_maxit;
+        for (int k = 0; k < n && closed; ++k) {
+            // the step's tangent in closed form (Solver::tangent_step): B = Z_{k+1} Z_k, the
+            // factors E+- (A1, RHS), G^T = 2 Z1 + (Z1 E-)^T (P), Z1' = sym(G^T + 1/2 G^T E+)
+            std::vector<GemmSpec> gb, g1, g2;
+            std::vector<GrpEw> dt, dsym;
+            std::vector<char> hp(G, 0);
+            bool any_hp = false;
+            for (int i = 0; i < G; ++i) {
+                Sys& sy = b->sys[i];
+                Mat* Z1 = (k % 2 == 0) ? &sy.Z1a : &sy.Z1b;
+                Mat* Z1n = (k % 2 == 0) ? &sy.Z1b : &sy.Z1a;
+                const int rows = D * sy.N;
+                hp[i] = mixed && sy.khp < n && k >= sy.khp - 2;
+                any_hp = any_hp || hp[i];
+                GemmSpec e;
+                e.skip = nullptr;
+                if (!hp[i]) {
+                    e.X = &sy.Z[k + 1];
+                    e.rows = sy.N;
+                    e.Y = &sy.Z[k];
+                    e.p = epi(sy.S.x, sy.N, sy.N, sy.ld);
+                    e.p.sym = 1;
+                    gb.push_back(e);
+                    add_flops(b, sym_flops(b, sy.N));
+                }
+                GrpEw t = ewd(sy.A1.hi, sy.A1.lo, sy.RHS.hi, sy.RHS.lo);
+                t.p4 = sy.Z[k + 1].x;
+                t.p5 = sy.S.x;
+                t.rows = sy.N; t.ld = sy.ld; t.N = sy.N; t.count = (long long)sy.blk;
+                dt.push_back(t);
+                e.X = Z1;
+                e.rows = rows;
+                e.Y = &sy.A1;
+                e.p = epi(sy.P.x, rows, sy.N, sy.ld, 1.f, 2.f, Z1->x);
+                e.p.trans_block = sy.N;
+                e.p.Dhi = sy.P.hi;
+                e.p.Dlo = sy.P.lo;
+                g1.push_back(e);
+                e.X = &sy.P;
+                e.Y = &sy.RHS;
+                e.p = epi(Z1n->x, rows, sy.N, sy.ld, 0.5f, 1.f, sy.P.x);
+                g2.push_back(e);
+                GrpEw y = ewd(Z1n->x, nullptr, Z1n->hi, Z1n->lo);
+                y.rows = rows; y.ld = sy.ld; y.N = sy.N;
+                dsym.push_back(y);
+                add_flops(b, 4.0 * D * (double)sy.N * sy.N * sy.N);
+            }
+            if (any_hp) CDMPT_TRY(step_product_hp(b, k, hp));
+            CDMPT_TRY(grouped_gemm(b, gb));
+            CDMPT_TRY(hp_join_lanes(b));
+            CDMPT_TRY(run_ew(b, G_TANGENT, dt));
+            CDMPT_TRY(grouped_gemm(b, g1));
+            CDMPT_TRY(grouped_gemm(b, g2));
+            CDMPT_TRY(run_tiles(b, dsym, D, grouped_symmetrize));
+        }
+        for (int k = 0; k < n && !closed; ++k) {
             std::vector<GemmSpec> gs, g1, g2;
             std::vector<GrpEw> dta, dz, dsym;
             std::vector<BCg> cg(G);
@@ -1598,6 +1909,10 @@ cdmpt_status cdmpt_batch_solve(cdmpt_batch* b, const double* beta, const double*
                 const double trQ = 0.25 * sy.beta * b->pinned[i * kSlots + B_TRQ];
                 for (int dd = 0; dd < D; ++dd) {
                     const double trP1 = 0.5 * b->pinned[i * kSlots + B_TRZ1 + dd];
+                    if (closed && !std::isfinite(trP1))
+                        return bfail_msg(b, CDMPT_ERR_CG_MAXITER,
+                                         "batch: the response met a non-finite value: no solution "
+                                         "of its linear systems");
                     const double m1 = trQ > 0 ? -trP1 / trQ : 0.0;
                     if (mu1) mu1[i * D + dd] = m1;
                     GrpEw a = ewd(Z1->x + (size_t)dd * sy.blk, sy.Qmu.x);

@@ -24,6 +24,22 @@ __device__ __forceinline__ void split1(float v, float* hi, float* lo, size_t i) 
     lo[i] = __uint_as_float(l);
 }
 
+__device__ __forceinline__ void split4(float a, float b, float c, float e, float* hi, float* lo,
+                                       size_t i) {
+    const float v[4] = {a, b, c, e};
+    float h[4], l[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        uint32_t hb, lb;
+        asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(hb) : "f"(v[k]));
+        h[k] = __uint_as_float(hb);
+        asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(lb) : "f"(v[k] - h[k]));
+        l[k] = __uint_as_float(lb);
+    }
+    *(float4*)(hi + i) = make_float4(h[0], h[1], h[2], h[3]);
+    *(float4*)(lo + i) = make_float4(l[0], l[1], l[2], l[3]);
+}
+
 __device__ __forceinline__ void block_add(double v, double* out) {
     __shared__ double part[32];
 #pragma unroll
@@ -174,6 +190,10 @@ __global__ void k_grouped(const GrpEw* __restrict__ desc) {
                 split1(x.w, d.p2, d.p3, i + 3);
             } else if constexpr (OP == G_ZERO) {
                 *(float4*)(d.p0 + i) = make_float4(0.f, 0.f, 0.f, 0.f);
+            } else if constexpr (OP == G_TANGENT) {
+                const float4 y = *(const float4*)(d.p4 + i), q = *(const float4*)(d.p5 + i);
+                split4(-y.x - q.x, -y.y - q.y, -y.z - q.z, -y.w - q.w, d.p0, d.p1, i);
+                split4(y.x - q.x, y.y - q.y, y.z - q.z, y.w - q.w, d.p2, d.p3, i);
             }
         }
     }
@@ -268,6 +288,28 @@ __global__ void k_grouped_tiles(const GrpEw* __restrict__ desc, int max_blocks) 
                 }
             }
         }
+    } else if constexpr (OP == 3) {   // pair (p0, p1) += (p4 + p4^T) / 2, as k_pair_add_sym
+        if (bi > bj) return;
+        const int x = threadIdx.x;
+        for (int y = threadIdx.y; y < TT; y += blockDim.y) {
+            a[y][x] = (i0 + y < N && j0 + x < N) ? d.p4[base + (size_t)(i0 + y) * ld + j0 + x] : 0.f;
+            b[y][x] = (j0 + y < N && i0 + x < N) ? d.p4[base + (size_t)(j0 + y) * ld + i0 + x] : 0.f;
+        }
+        __syncthreads();
+        auto put_one = [&](int r, int c, float v) {
+            if (r >= N || c >= N) return;
+            const size_t i = base + (size_t)r * ld + c;
+            float h, l;
+            dd::add1(d.p0[i], d.p1[i], v, h, l);
+            d.p0[i] = h;
+            d.p1[i] = l;
+            if (d.p2) split1(h, d.p2, d.p3, i);
+        };
+#pragma unroll 4
+        for (int y = threadIdx.y; y < TT; y += blockDim.y) {
+            put_one(i0 + y, j0 + x, 0.5f * (a[y][x] + b[x][y]));
+            if (bi != bj) put_one(j0 + y, i0 + x, 0.5f * (a[x][y] + b[y][x]));
+        }
     } else {                   // p0 = p1 + p1^T
         for (int y = threadIdx.y; y < TT; y += blockDim.y) {
             const int r = j0 + y, c = i0 + threadIdx.x;
@@ -282,6 +324,58 @@ __global__ void k_grouped_tiles(const GrpEw* __restrict__ desc, int max_blocks) 
                 d.p0[i] = v;
                 if (d.p2) split1(v, d.p2, d.p3, i);
             }
+        }
+    }
+}
+
+// Coefficient blocks of a matrix polynomial, one pass over the powers (k_poly_blocks).
+template <int NP, int NB>
+__global__ void k_grouped_poly(const GrpPoly* __restrict__ desc) {
+    const GrpPoly& d = desc[blockIdx.y];
+    if (d.skip && *d.skip != 0.0) return;
+    const float* P[NP];
+    float* out[NB];
+    float k[NB][NP + 1];
+#pragma unroll
+    for (int j = 0; j < NP; ++j) P[j] = d.P[j];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        out[b] = d.out[b];
+#pragma unroll
+        for (int j = 0; j <= NP; ++j) k[b][j] = d.coef[b][j];
+    }
+    float* const hi = d.hi;
+    float* const lo = d.lo;
+    const float c = d.c;
+    const size_t nv = (size_t)d.count / 4, lv = (size_t)d.ld / 4;
+    for (size_t v = blockIdx.x * (size_t)blockDim.x + threadIdx.x; v < nv;
+         v += (size_t)gridDim.x * blockDim.x) {
+        const size_t r = v / lv;
+        const int g = (int)r - (int)(v - r * lv) * 4;   // diagonal position inside the vector
+        float x[NP][4];
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+            const float4 t = *(const float4*)(P[j] + v * 4);
+            x[j][0] = t.x;
+            x[j][1] = t.y;
+            x[j][2] = t.z;
+            x[j][3] = t.w;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (g == i) x[0][i] -= c;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            float y[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                y[i] = k[b][1] * x[0][i];
+#pragma unroll
+                for (int j = 1; j < NP; ++j) y[i] = fmaf(k[b][j + 1], x[j][i], y[i]);
+                if (g == i) y[i] += k[b][0];
+            }
+            *(float4*)(out[b] + v * 4) = make_float4(y[0], y[1], y[2], y[3]);
+            if (b == NB - 1) split4(y[0], y[1], y[2], y[3], hi, lo, v * 4);
         }
     }
 }
@@ -359,6 +453,7 @@ cdmpt_status grouped_ew(int op, const GrpEw* dev_desc, int G, long long max_coun
         case G_PAIR_INIT: k_grouped<G_PAIR_INIT><<<grid, kT, 0, s>>>(dev_desc); break;
         case G_PAIR_LINCOMB: k_grouped<G_PAIR_LINCOMB><<<grid, kT, 0, s>>>(dev_desc); break;
         case G_PAIR_ADD: k_grouped<G_PAIR_ADD><<<grid, kT, 0, s>>>(dev_desc); break;
+        case G_TANGENT: k_grouped<G_TANGENT><<<grid, kT, 0, s>>>(dev_desc); break;
         default: set_error("grouped_ew: unknown op"); return CDMPT_ERR_ARG;
     }
     return check("grouped elementwise launch");
@@ -386,6 +481,35 @@ cdmpt_status grouped_pair_symmetrize(const GrpEw* dev_desc, int G, int max_N, in
     dim3 grid(nt, nt, G * max_blocks), block(TT, 8);
     k_grouped_tiles<2><<<grid, block, 0, s>>>(dev_desc, max_blocks);
     return check("grouped pair symmetrize launch");
+}
+
+cdmpt_status grouped_pair_add_sym(const GrpEw* dev_desc, int G, int max_N, int max_blocks,
+                                  cudaStream_t s) {
+    const int nt = (max_N + TT - 1) / TT;
+    dim3 grid(nt, nt, G * max_blocks), block(TT, 8);
+    k_grouped_tiles<3><<<grid, block, 0, s>>>(dev_desc, max_blocks);
+    return check("grouped pair correction launch");
+}
+
+cdmpt_status grouped_poly(const GrpPoly* dev_desc, int G, int np, int nb, long long max_count,
+                          cudaStream_t s) {
+    if (G <= 0) return CDMPT_OK;
+    const long long work = std::max<long long>(1, max_count / 4);
+    dim3 grid((unsigned)std::min<long long>(64, (work + kT - 1) / kT), G);
+    auto is = [&](int a, int c) { return np == a && nb == c; };
+    if (is(2, 1))
+        k_grouped_poly<2, 1><<<grid, kT, 0, s>>>(dev_desc);
+    else if (is(3, 3))
+        k_grouped_poly<3, 3><<<grid, kT, 0, s>>>(dev_desc);
+    else if (is(3, 4))
+        k_grouped_poly<3, 4><<<grid, kT, 0, s>>>(dev_desc);
+    else if (is(4, 4))
+        k_grouped_poly<4, 4><<<grid, kT, 0, s>>>(dev_desc);
+    else {
+        set_error("grouped matrix polynomial: no kernel for this block shape");
+        return CDMPT_ERR_ARG;
+    }
+    return check("grouped matrix polynomial launch");
 }
 
 cdmpt_status grouped_trace(const GrpEw* dev_desc, int G, int max_N, int max_blocks,

@@ -23,7 +23,23 @@ struct GrpEw {
     double s0, s1;        // op coefficients
     const double* skip;   // system skipped while *skip != 0 (may be null)
     double s2;            // CG init: tolerance^2 on the reference norm in slot kCgRefSlot (0: none)
+    float* p5;            // G_TANGENT only
 };
+
+// Per-system operands of the coefficient blocks of a matrix polynomial (Ew<T>::PolyBlocks).
+struct GrpPoly {
+    const float* P[4];    // W, S^2, S^3, S^4
+    float* out[4];
+    float* hi;            // split of the last block
+    float* lo;
+    float c;
+    float coef[4][5];
+    long long count;
+    int ld;
+    const double* skip;
+};
+cdmpt_status grouped_poly(const GrpPoly* dev_desc, int G, int np, int nb, long long max_count,
+                          cudaStream_t s);
 
 // Per-system scalar slot that holds ||ref||^2 of a CG solve's absolute tolerance.
 constexpr int kCgRefSlot = 11;
@@ -42,6 +58,8 @@ enum GrpOp {
     G_PAIR_INIT = 9,      // (p0, p1) = s0 (h - s1 I) rounded to a pair, split of p0 to (p2, p3)
     G_PAIR_LINCOMB = 10,  // p0 = FP32(s0 (p1 + p2) + s1 (p3 + p4)), s0 and s1 powers of two
     G_PAIR_ADD = 11,      // (p0, p1) += p2 without rounding to FP32, split of p0 to (p3, p4)
+    // factors of a step's tangent map: (p0, p1) = split(-p4 - p5), (p2, p3) = split(p4 - p5)
+    G_TANGENT = 12,
 };
 
 cdmpt_status grouped_ew(int op, const GrpEw* dev_desc, int G, long long max_count,
@@ -56,6 +74,9 @@ cdmpt_status grouped_trace(const GrpEw* dev_desc, int G, int max_N, int max_bloc
 // (p0, p1) = ((p0, p1) + (p0, p1)^T) / 2 for pair-stored blocks, split of p0 to (p2, p3)
 cdmpt_status grouped_pair_symmetrize(const GrpEw* dev_desc, int G, int max_N, int max_blocks,
                                      cudaStream_t s);
+// pair (p0, p1) += (p4 + p4^T) / 2, split of p0 to (p2, p3)
+cdmpt_status grouped_pair_add_sym(const GrpEw* dev_desc, int G, int max_N, int max_blocks,
+                                  cudaStream_t s);
 // CG scalar steps: one thread per system; init also sets done for skipped systems
 cdmpt_status grouped_cg_init(const GrpEw* dev_desc, int G, cudaStream_t s);
 cdmpt_status grouped_cg_step(const GrpEw* dev_desc, int G, cudaStream_t s);

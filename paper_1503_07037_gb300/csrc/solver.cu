@@ -837,7 +837,8 @@ cdmpt_status Solver<T>::tanh_taylor(Context& cx, int m) {
 // cut after degree m with an error below 2 q^(m+1) / (g (1 - q)); near-minimax. For [0, 1]
 // and x0 = 1, q = 0.17: degree 9 for 1e-7, 18 for 1e-14. The shapes (s, r) below are the ones
 // with the fewest products s - 1 + r for their degree; a shape's whole degree is used.
-bool InversePoly::fit(double x0, double lo, double hi, double tol, int max_degree) {
+bool InversePoly::fit(double x0, double lo, double hi, double tol, int max_degree, int want_s,
+                      int want_r) {
     static const int shape[][2] = {{1, 0}, {2, 0}, {2, 1}, {2, 2}, {3, 2}, {3, 3}, {4, 3}, {5, 3}};
     s = r = 0;
     const double h = 0.5 * (hi - lo), A = x0 + 0.5 * (hi + lo);
@@ -850,7 +851,8 @@ bool InversePoly::fit(double x0, double lo, double hi, double tol, int max_degre
         err *= q;
     }
     for (const auto& sh : shape)
-        if (sh[0] * (sh[1] + 1) >= need && sh[0] * (sh[1] + 1) <= kMaxDegree) {
+        if (sh[0] * (sh[1] + 1) >= need && sh[0] * (sh[1] + 1) <= kMaxDegree &&
+            (want_s == 0 || (sh[0] == want_s && sh[1] == want_r))) {
             s = sh[0];
             r = sh[1];
             break;
@@ -1403,7 +1405,7 @@ cdmpt_status Solver<T>::compute_q(Context& cx) {
 
 // Largest Krylov degree any step's solve needs at relative tolerance tol: the spectrum of A_k
 // lies in [1, 2], on which m CG iterations gain 2 q^m, q = (sqrt(2) - 1) / (sqrt(2) + 1).
-static int krylov_degree(double tol) {
+int krylov_degree(double tol) {
     return (int)std::ceil(std::log(std::max(tol, 1e-300) / 2.0) / std::log(0.17157));
 }
 

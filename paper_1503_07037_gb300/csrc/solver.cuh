@@ -69,9 +69,14 @@ struct InversePoly {
     double a[kMaxDegree + 1] = {};
     int degree() const { return s * (r + 1); }
     // Relative error (x0 + w) |p - 1 / (x0 + w)| <= tol on [lo, hi], degree <= max_degree;
-    // false (s = 0) if that takes a higher degree
-    bool fit(double x0, double lo, double hi, double tol, int max_degree);
+    // false (s = 0) if that takes a higher degree. want_s > 0: of the shape (want_s, want_r),
+    // false if its degree is too low
+    bool fit(double x0, double lo, double hi, double tol, int max_degree, int want_s = 0,
+             int want_r = 0);
 };
+
+// Largest Krylov degree a step's solve needs at relative tolerance tol (see solver.cu)
+int krylov_degree(double tol);
 
 template <typename T>
 class Solver {
