@@ -227,45 +227,42 @@ __device__ __forceinline__ void st8(uint32_t ta, const int* v) {
                  : "memory");
 }
 
-// FP64 value of (J 2^16 + T) 2^e, rounded to nearest even. Integer operations only, but for
-// results outside the normal range.
-__device__ __forceinline__ double oz64_value(long long J, long long T, int e) {
+// FP64 value of (J 2^16 + T) 2^e, rounded to nearest even, by integer operations without a
+// branch, so that the eight columns of an epilogue chunk interleave (with branches each
+// element waited for its own chain of about a hundred operations: 1400 clocks per column,
+// 23 us of a 128-row product's 37). *odd: the value is outside the normal range.
+__device__ __forceinline__ double oz64_value(long long J, long long T, int e, bool* odd) {
     unsigned long long lo = (unsigned long long)J << 16;
-    long long hi = J >> 48;
+    unsigned long long hi = (unsigned long long)(J >> 48);
     const unsigned long long sum = lo + (unsigned long long)T;
-    hi += (T >> 63) + (sum < lo ? 1 : 0);
-    lo = sum;
-    const bool neg = hi < 0;
-    if (neg) {
-        lo = 0ull - lo;
-        hi = ~hi + (lo == 0ull ? 1 : 0);
-    }
-    unsigned long long h = (unsigned long long)hi;
-    if ((h | lo) == 0ull) return 0.0;
-    int lz;
-    if (h == 0ull) {
-        const int l = __clzll((long long)lo);
-        h = lo << l;
-        lo = 0ull;
-        lz = 64 + l;
-    } else {
-        lz = __clzll((long long)h);
-        if (lz > 0) {
-            h = (h << lz) | (lo >> (64 - lz));
-            lo <<= lz;
-        }
-    }
+    hi += (unsigned long long)(T >> 63) + (unsigned long long)(sum < lo);
+    const unsigned long long neg = (unsigned long long)((long long)hi >> 63);   // all ones: negative
+    lo = sum ^ neg;
+    hi ^= neg;
+    lo -= neg;
+    hi += (unsigned long long)(neg != 0ull && lo == 0ull);
+    // normalise: the leading one to bit 127
+    const bool small = hi == 0ull;
+    const int l = __clzll((long long)(small ? lo : hi));   // 64 if both are zero
+    const int s = l & 63;
+    const unsigned long long h0 = small ? lo : hi, l0 = small ? 0ull : lo;
+    const unsigned long long h = (h0 << s) | ((l0 >> 1) >> (63 - s));
+    const unsigned long long r = l0 << s;
     unsigned long long m = h >> 11;   // 53 bits, the leading one at bit 52
     const unsigned long long rest = h & 0x7ffull;
-    if (rest > 0x400ull || (rest == 0x400ull && (lo != 0ull || (m & 1ull)))) ++m;
-    const int be = 1023 + 127 - lz + e;
-    if (be >= 1 && be <= 2045) {
-        const unsigned long long b = ((unsigned long long)be << 52) + (m - (1ull << 52)) +
-                                     (neg ? 1ull << 63 : 0ull);
-        return __longlong_as_double((long long)b);
-    }
-    const double v = ldexp((double)m, 75 - lz + e);
-    return neg ? -v : v;
+    m += (unsigned long long)(rest > 0x400ull || (rest == 0x400ull && (r != 0ull || (m & 1ull))));
+    const int be = 1023 + 127 - l - (small ? 64 : 0) + e;
+    const bool zero = h0 == 0ull;
+    *odd = !zero && (be < 1 || be > 2045);
+    const unsigned long long b = ((unsigned long long)(unsigned)be << 52) + (m - (1ull << 52)) +
+                                 (neg & (1ull << 63));
+    return __longlong_as_double((long long)(zero ? 0ull : b));
+}
+
+// The same value in general, for results outside the normal range.
+__device__ __noinline__ double oz64_value_odd(long long J, long long T, int e) {
+    // J and T apart: the sum of two scaled doubles rounds once where the result is normal
+    return ldexp((double)J, e + 16) + ldexp((double)T, e);
 }
 
 // Tile t of a launch: row-tile fastest, or, for a symmetric result, over the tiles whose 64
@@ -498,6 +495,9 @@ __global__ void __launch_bounds__(Z_THREADS, 1)
             tmem_wait_st();
             const bool row_ok = m < p.M;
             const int ex = row_ok ? ex_[m] : 0;
+            const int mdiag = p.gamma != 0.0 ? m % p.diag_block : -1;
+            const int tb = p.trans_block > 0 ? m / p.trans_block : 0;
+            const size_t trow = (size_t)tb * p.trans_block, tcol = (size_t)(m - tb * p.trans_block);
 #pragma unroll 1
             for (int c0 = 0; c0 < Z_CW; c0 += 8) {
                 uint32_t r[Z_NG][8];
@@ -513,34 +513,73 @@ __global__ void __launch_bounds__(Z_THREADS, 1)
                     for (int j = 0; j < 8; ++j) {
                         const int n = n0 + c0 + j;
                         const bool ok = n < p.N && !(p.sym && n < m);
-                        size_t rr, cc;
-                        epi_position(p, m, n, rr, cc);
+                        const size_t rr = p.trans_block > 0 ? trow + n : (size_t)m;
+                        const size_t cc = p.trans_block > 0 ? tcol : (size_t)n;
                         eyv[j] = ok ? ey_[n] : 0;
                         cv[j] = (ok && p.beta != 0.0) ? p.C[rr * p.ldc + cc] : 0.0;
                         ev[j] = (ok && p.dot && p.E) ? p.E[rr * p.lde + cc] : 0.0;
                     }
+                    double val[8];
+                    unsigned odd = 0u;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        long long J = 0;
+#pragma unroll
+                        for (int g = 0; g < Z_NX; ++g) J = J * 256 + (long long)(int)r[g][j];
+                        J = J * 256 + (long long)__float2int_rn(__uint_as_float(r[Z_NX][j]));
+                        const long long T =
+                            (long long)__float2int_rn(__uint_as_float(r[Z_NX + 1][j])) * 256 +
+                            (long long)__float2int_rn(__uint_as_float(r[Z_NX + 2][j]));
+                        bool o;
+                        val[j] = oz64_value(J, T, ex + eyv[j] + alpha_exp - 62, &o);
+                        if (o) odd |= 1u << j;
+                    }
+                    if (odd) {
+#pragma unroll 1
+                        for (int j = 0; j < 8; ++j) {
+                            if (!(odd >> j & 1u)) continue;
+                            long long J = 0, T = 0;
+                            int q8 = 0;
+                            double x = 0.0;
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {   // register arrays: no dynamic index
+                                if (i != j) continue;
+#pragma unroll
+                                for (int g = 0; g < Z_NX; ++g)
+                                    J = J * 256 + (long long)(int)r[g][i];
+                                J = J * 256 +
+                                    (long long)__float2int_rn(__uint_as_float(r[Z_NX][i]));
+                                T = (long long)__float2int_rn(__uint_as_float(r[Z_NX + 1][i])) *
+                                        256 +
+                                    (long long)__float2int_rn(__uint_as_float(r[Z_NX + 2][i]));
+                                q8 = eyv[i];
+                            }
+                            x = oz64_value_odd(J, T, ex + q8 + alpha_exp - 62);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                if (i == j) val[i] = x;
+                        }
+                    }
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         const int n = n0 + c0 + j;
-                        if (n < p.N && !(p.sym && n < m)) {
-                            long long J = 0;
+                        double v = alpha_neg < 0 ? p.alpha * val[j] : (alpha_neg ? -val[j] : val[j]);
+                        if (p.beta != 0.0) v = fma(p.beta, cv[j], v);
+                        if (p.gamma != 0.0 && mdiag == n) v += p.gamma;
+                        val[j] = v;
+                    }
 #pragma unroll
-                            for (int g = 0; g < Z_NX; ++g) J = J * 256 + (long long)(int)r[g][j];
-                            J = J * 256 + (long long)__float2int_rn(__uint_as_float(r[Z_NX][j]));
-                            const long long T =
-                                (long long)__float2int_rn(__uint_as_float(r[Z_NX + 1][j])) * 256 +
-                                (long long)__float2int_rn(__uint_as_float(r[Z_NX + 2][j]));
-                            double v = oz64_value(J, T, ex + eyv[j] + alpha_exp - 62);
-                            v = alpha_neg < 0 ? p.alpha * v : (alpha_neg ? -v : v);
-                            size_t rr, cc;
-                            epi_position(p, m, n, rr, cc);
-                            if (p.beta != 0.0) v = fma(p.beta, cv[j], v);
-                            if (p.gamma != 0.0 && (m % p.diag_block) == n) v += p.gamma;
-                            p.D[rr * p.ldd + cc] = v;
-                            const bool mirror = p.sym && n != m;
-                            if (mirror) p.D[(size_t)n * p.ldd + m] = v;
-                            if (p.dot) dsum += v * (p.E ? ev[j] : v) * (mirror ? 2.0 : 1.0);
+                    for (int j = 0; j < 8; ++j) {
+                        const int n = n0 + c0 + j;
+                        const bool ok = n < p.N && !(p.sym && n < m);
+                        const bool mirror = p.sym && n != m;
+                        const size_t o = p.trans_block > 0 ? (trow + n) * p.ldd + tcol
+                                                           : (size_t)m * p.ldd + n;
+                        if (ok) {
+                            p.D[o] = val[j];
+                            if (mirror) p.D[(size_t)n * p.ldd + m] = val[j];
                         }
+                        if (p.dot && ok) dsum += val[j] * (p.E ? ev[j] : val[j]) * (mirror ? 2.0 : 1.0);
                     }
                 }
             }
