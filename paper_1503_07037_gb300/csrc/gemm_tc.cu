@@ -47,6 +47,7 @@
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
@@ -696,16 +697,31 @@ cdmpt_status launch(int M, int N, int K, const float* X, const float* Xl, int ld
     return CDMPT_OK;
 }
 
-// Kernel family for single (non-grouped) products with more than 128 rows: one SM per
-// tile or the two-SM MMA (cta_group::2, 256 x 256 tiles; for split TF32 the wide kernel
-// k_gemm_split2sm). Default: two-SM for both; CDMPT_TC_MODE=1sm|2sm forces one family.
-bool use_2sm(bool /*three*/) {
+// Kernel family for single (non-grouped) products with more than 128 rows: 128 x 128 tiles on
+// one SM, or 256 x 256 tiles on an SM pair (cta_group::2; for split TF32 the wide kernel
+// k_gemm_split2sm). Both take about the same time per tile and k (split 25 ns, one-pass 9 ns),
+// the pair's tile having twice the work per SM, and a fixed part that the larger tile's
+// epilogue lengthens (in units of k: split 330 and 590; one-pass 700 and 1000). So the small tile
+// wins where its tiles still fit one wave or the pairs' tiles leave SMs idle, and the line is
+// drawn by the waves of either. Measured, split, one SM against two: N = 512 21 and 28 us,
+// 1536 46 and 54, 2048 107 and 68 (63 and 70 for a symmetric result), 4096 687 and 477.
+// CDMPT_TC_MODE=1sm|2sm forces one family.
+bool use_2sm(bool three, int M, int N, int K, bool sym) {
     static int v = -2;
     if (v == -2) {
         const char* e = getenv("CDMPT_TC_MODE");
         v = !e ? -1 : (std::strcmp(e, "2sm") == 0 ? 1 : 0);
     }
-    return v != 0;
+    if (v >= 0) return v == 1;
+    auto waves = [&](int t, int slots) {
+        const long long mt = (M + t - 1) / t, nt = (N + t - 1) / t;
+        const long long tiles = sym ? mt * (mt + 1) / 2 : mt * nt;
+        return (double)((tiles + slots - 1) / slots);
+    };
+    const int sms = sm_count();
+    const double one = waves(BM, sms) * (K + (three ? 330 : 700));
+    const double two = waves(2 * BM, std::max(1, sms / 2)) * (K + (three ? 590 : 1000));
+    return two < one;
 }
 
 template <int BN, int STAGES, int PASSES, int KCH>
@@ -910,25 +926,11 @@ cdmpt_status gemm_tc_f32(int engine, int M, int N, int K, const Operand<float>& 
             default: return launch<128, 3, 3, 2, true>(M, N, K, xh, X.lo, ldx, yh, Y.lo, ldy, p, skip, s, screen);
         }
     }
-    if (p.sym) {
-        // symmetric result: square tiles, upper triangle only (256 x 256 two-SM tiles; split
-        // TF32 on one-SM 128 x 128 tiles when M <= 128 or the one-SM family is forced)
-        if (!three)
-            return gemm_tc_2sm(false, 0, M, N, K, xh, xh, ldx, yh, yh, ldy, p, skip, s);
-        if (use_2sm(true) && M > BM)
-            return gemm_tc_2sm(true, split_chunk(), M, N, K, xh, X.lo, ldx, yh, Y.lo, ldy, p,
-                               skip, s);
-        switch (split_chunk()) {
-            case 1: return launch<128, 3, 3, 1>(M, N, K, xh, X.lo, ldx, yh, Y.lo, ldy, p, skip, s);
-            case 4: return launch<128, 3, 3, 4>(M, N, K, xh, X.lo, ldx, yh, Y.lo, ldy, p, skip, s);
-            case 0: return launch<128, 3, 3, 0>(M, N, K, xh, X.lo, ldx, yh, Y.lo, ldy, p, skip, s);
-            default: return launch<128, 3, 3, 2>(M, N, K, xh, X.lo, ldx, yh, Y.lo, ldy, p, skip, s);
-        }
-    }
-    if (use_2sm(three) && M > BM)
-        return gemm_tc_2sm(three, split_chunk(), M, N, K, xh, three ? X.lo : xh, ldx, yh, three ? Y.lo : yh,
-                           ldy, p, skip, s);
-    if (!three) return launch<256, 4, 1, 0>(M, N, K, xh, xh, ldx, yh, yh, ldy, p, skip, s);
+    // symmetric results need square tiles: upper triangle only
+    if (M > BM && use_2sm(three, M, N, K, p.sym != 0))
+        return gemm_tc_2sm(three, split_chunk(), M, N, K, xh, three ? X.lo : xh, ldx, yh,
+                           three ? Y.lo : yh, ldy, p, skip, s);
+    if (!three) return launch<128, 6, 1, 0>(M, N, K, xh, xh, ldx, yh, yh, ldy, p, skip, s);
     switch (split_chunk()) {
         case 1: return launch<128, 3, 3, 1>(M, N, K, xh, X.lo, ldx, yh, Y.lo, ldy, p, skip, s);
         case 4: return launch<128, 3, 3, 4>(M, N, K, xh, X.lo, ldx, yh, Y.lo, ldy, p, skip, s);

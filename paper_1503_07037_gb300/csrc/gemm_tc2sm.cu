@@ -447,8 +447,9 @@ __global__ void __launch_bounds__(Cfg2<BN, STAGES, PASSES>::THREADS, 1)
 // (about 0.9 us at the TF32 rate); its arrival on the peer's barrier uses the plain
 // (.release.cta) form, since a cluster-scope release made every drain wait for the previous
 // tile's global stores (ncu: membar stalls dominated, 232 TF/s at N = 8192 against 344
-// without). A finished tile is stored from the registers in 32 x 32 blocks through the warp's
-// shared-memory transpose buffer (tc_store.cuh); the MMA meanwhile fills the other accumulator. Tiles run in groups of eight M-tiles (grouped raster), or over the
+// without). A finished tile goes back to the accumulator last drained and from there in 32 x 32 blocks
+// through the warp's shared-memory transpose buffer (tc_store.cuh); the MMA meanwhile fills the
+// other accumulator. Tiles run in groups of eight M-tiles (grouped raster), or over the
 // upper triangle for symmetric results.
 constexpr int SPLIT_BN = 256;
 constexpr int SPLIT_GROUP = 8;
@@ -753,16 +754,34 @@ __global__ void __launch_bounds__(split_threads(EW), 1)
 #pragma unroll
                     for (int j = 0; j < LW; ++j) acc[c0 + j] += __uint_as_float(rr[j]);
                 }
+                if (c + 1 == nch) break;   // the last chunk's columns take the sums (below)
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_remote(tempty0 + (uint32_t)b * 8u);
             }
             if (!ok) break;
+            // The finished sums go back to this warp's columns of the accumulator just drained
+            // and are stored from there block by block: the store code then has the registers
+            // to itself (beside 128 live sums it spilled or ran element by element) and stands
+            // once. The MMAs of the next tile start on the other accumulator meanwhile.
+            const int b = g % NB;
+            ++g;
 #pragma unroll
+            for (int c0 = 0; c0 < CW; c0 += 32)
+                tmem_st32(lane_base + (uint32_t)(b * BN + c0), acc + c0);
+            tmem_wait_st();
+#pragma unroll 1
             for (int c0 = 0; c0 < CW; c0 += 32) {
+                uint32_t rr[32];
+                tmem_ld32(lane_base + (uint32_t)(b * BN + c0), rr);
+                if (c0 + 32 >= CW) {   // all read: the accumulator is free again
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_remote(tempty0 + (uint32_t)b * 8u);
+                }
                 float a[32];
 #pragma unroll
-                for (int j = 0; j < 32; ++j) a[j] = acc[c0 + j];
+                for (int j = 0; j < 32; ++j) a[j] = __uint_as_float(rr[j]);
                 dsum += (double)epi_block32(P, m - lane, n0 + c0, diag, a, xbuf, lane);
             }
             if constexpr (GROUPED) {

@@ -12,9 +12,15 @@
 // rows are the block's columns: those stores are row segments as well.
 //
 // A single warp per scheduler runs this code while the tensor pipe works, so it is written
-// for few instructions and no divergent branches: the symmetric mirror and the TF32 split
-// copies are template parameters chosen once per tile, beta C, gamma I and the dot enter
-// through selects, and out-of-range elements are masked by predicated stores.
+// for few instructions: two warps per scheduler execute straight-line code at about one
+// instruction in eight clocks (the stall is instruction fetch), and the element-wise form of a
+// block, about a thousand instructions, took 8000 clocks whether or not it stored anything;
+// four such blocks were 17 of the 35 us of a 256 x 256 tile at K = 512. Blocks off
+// the diagonal and with 16-byte rows therefore move four elements per instruction
+// (epi_block32_vec, epi_block32_trans_vec); the other blocks take the masked element-wise form,
+// where the symmetric mirror and the TF32 split copies are template parameters chosen once per
+// tile, beta C, gamma I and the dot enter through selects, and out-of-range elements are
+// masked by predicated stores.
 #pragma once
 
 #include <cstdint>
@@ -24,9 +30,14 @@
 namespace cdmpt {
 namespace tc {
 
-// Words of one warp's transpose buffer: 32 rows of 33, the pad word keeping both the
-// row-wise and the column-wise passes free of bank conflicts.
+// Words of one warp's transpose buffer: 32 rows of 33 for the element-wise form, the pad word
+// keeping both the row-wise and the column-wise passes free of bank conflicts. The
+// four-element form takes 32 rows of 32 words whose 16-byte chunk j stands at j ^ (row % 8), so
+// that eight lanes cover all banks once along a row and down a column of chunks.
 constexpr int kXposeWords = 32 * 33;
+__device__ __forceinline__ int xpose_at(int row, int chunk) {
+    return row * 32 + 4 * (chunk ^ (row & 7));
+}
 
 __device__ __forceinline__ void split_tf32(float v, float& h, float& l) {
     uint32_t hb, lb;
@@ -177,6 +188,205 @@ __device__ __forceinline__ float epi_block32_trans(const EpiParams<float>& p, in
     return local;
 }
 
+// Four elements' TF32 split, stored.
+__device__ __forceinline__ void split_tf32_x4(const float4& v, float* hi, float* lo) {
+    float4 h, l;
+    split_tf32(v.x, h.x, l.x);
+    split_tf32(v.y, h.y, l.y);
+    split_tf32(v.z, h.z, l.z);
+    split_tf32(v.w, h.w, l.w);
+    *(float4*)hi = h;
+    *(float4*)lo = l;
+}
+
+// The block, off the diagonal of a symmetric result, arrays and leading dimensions 16-byte and
+// its columns inside the matrix a multiple of 4: lane l takes columns 4 (l % 8) of rows
+// l / 8 + 4 i, so a warp instruction moves four 128-byte row segments.
+template <bool SYM, bool SPLIT>
+__device__ __forceinline__ float epi_block32_vec(const EpiParams<float>& p, int m0, int n,
+                                                 float* S, int lane) {
+    constexpr int RB = 2;   // row groups whose loads are issued together
+    const size_t ldd = (size_t)p.ldd;
+    const float alpha = p.alpha, beta = p.beta, gamma = p.gamma;
+    const bool has_c = beta != 0.f, has_dot = p.dot != nullptr;   // E is null here
+    const int r0 = lane >> 3, c0 = (lane & 7) * 4;
+    // column of the diagonal of gamma I in row m0 + r0, relative to this lane's first column
+    int dg = gamma != 0.f ? (m0 + r0) % p.diag_block - (n + c0) : 1 << 30;
+    const int db = p.diag_block;
+    const size_t o0 = (size_t)(m0 + r0) * ldd + n + c0;
+    float* Dp = p.D + o0;
+    float* Hp = SPLIT ? p.Dhi + o0 : nullptr;
+    float* Lp = SPLIT ? p.Dlo + o0 : nullptr;
+    const float* Cp = has_c ? p.C + (size_t)(m0 + r0) * p.ldc + n + c0 : nullptr;
+    const size_t sd = 4 * ldd, sc = 4 * (size_t)p.ldc;
+    // rows r0 + 4 i: chunk l % 8 alternates between two places
+    const int rows = n + c0 < p.N ? p.M - m0 - r0 : 0;   // this lane's rows 4 i < rows exist
+    float* Sp = S + r0 * 32;
+    const int s0 = 4 * ((lane & 7) ^ r0), s1 = s0 ^ 16;
+    float local = 0.f;
+#pragma unroll 1
+    for (int i0 = 0; i0 < 8; i0 += RB) {
+        float4 v[RB], cv[RB];
+#pragma unroll
+        for (int i = 0; i < RB; ++i) {
+            if (has_c && 4 * (i0 + i) < rows) cv[i] = *(const float4*)(Cp + i * sc);
+            v[i] = *(const float4*)(Sp + i * 128 + ((i & 1) ? s1 : s0));
+        }
+#pragma unroll
+        for (int i = 0; i < RB; ++i) {
+            float4 w = v[i];
+            w.x *= alpha;
+            w.y *= alpha;
+            w.z *= alpha;
+            w.w *= alpha;
+            if (has_c) {
+                w.x = fmaf(beta, cv[i].x, w.x);
+                w.y = fmaf(beta, cv[i].y, w.y);
+                w.z = fmaf(beta, cv[i].z, w.z);
+                w.w = fmaf(beta, cv[i].w, w.w);
+            }
+            if ((unsigned)dg < 4u) {
+                w.x += dg == 0 ? gamma : 0.f;
+                w.y += dg == 1 ? gamma : 0.f;
+                w.z += dg == 2 ? gamma : 0.f;
+                w.w += dg == 3 ? gamma : 0.f;
+            }
+            dg += 4;
+            if (gamma != 0.f && dg + n + c0 >= db) dg -= db;
+            if constexpr (SYM) *(float4*)(Sp + i * 128 + ((i & 1) ? s1 : s0)) = w;
+            v[i] = w;
+            if (has_dot && 4 * (i0 + i) < rows)
+                local += w.x * w.x + w.y * w.y + w.z * w.z + w.w * w.w;
+        }
+#pragma unroll
+        for (int i = 0; i < RB; ++i) {
+            if (4 * (i0 + i) < rows) {
+                *(float4*)(Dp + i * sd) = v[i];
+                if constexpr (SPLIT) split_tf32_x4(v[i], Hp + i * sd, Lp + i * sd);
+            }
+        }
+        Dp += RB * sd;
+        if constexpr (SPLIT) {
+            Hp += RB * sd;
+            Lp += RB * sd;
+        }
+        Cp += has_c ? RB * sc : 0;
+        Sp += RB * 128;
+    }
+    if constexpr (SYM) {
+        // the mirrored block: lane l on row m0 + l, columns n + j to rows n + j
+        __syncwarp();
+        const size_t q0 = (size_t)n * ldd + m0 + lane;
+        float* Mp = p.D + q0;
+        float* Mh = SPLIT ? p.Dhi + q0 : nullptr;
+        float* Ml = SPLIT ? p.Dlo + q0 : nullptr;
+        const int cols = m0 + lane < p.M ? p.N - n : 0;   // rows n + j, j < cols, take this lane's
+#pragma unroll 1
+        for (int j = 0; j < 32; j += 8) {
+            const float4 a = *(const float4*)(S + xpose_at(lane, j >> 2)),
+                         b = *(const float4*)(S + xpose_at(lane, (j >> 2) + 1));
+            const float w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if (j + i >= cols) break;
+                Mp[i * ldd] = w[i];
+                if constexpr (SPLIT) {
+                    float h, l;
+                    split_tf32(w[i], h, l);
+                    Mh[i * ldd] = h;
+                    Ml[i * ldd] = l;
+                }
+            }
+            Mp += 8 * ldd;
+            if constexpr (SPLIT) {
+                Mh += 8 * ldd;
+                Ml += 8 * ldd;
+            }
+        }
+        local *= 2.f;   // the mirror counts too
+    }
+    return local;
+}
+
+// Transposed placement of a block inside one row block: lane l holds row m0 + l, so that the lanes write consecutive columns of each row n + j of the row block.
+template <bool SPLIT>
+__device__ __forceinline__ float epi_block32_trans_vec(const EpiParams<float>& p, int m0, int n,
+                                                       const float* S, int lane) {
+    const int b = m0 / p.trans_block;
+    const size_t r0 = (size_t)b * p.trans_block + n, c = (size_t)(m0 + lane - b * p.trans_block);
+    const size_t ldd = (size_t)p.ldd, ldc = (size_t)p.ldc;
+    const float alpha = p.alpha, beta = p.beta, gamma = p.gamma;
+    const bool has_c = beta != 0.f, has_dot = p.dot != nullptr;   // E is null here
+    const int md = gamma != 0.f ? (m0 + lane) % p.diag_block - n : -1;
+    float* Dp = p.D + r0 * ldd + c;
+    float* Hp = SPLIT ? p.Dhi + r0 * ldd + c : nullptr;
+    float* Lp = SPLIT ? p.Dlo + r0 * ldd + c : nullptr;
+    const float* Cp = has_c ? p.C + r0 * ldc + c : nullptr;
+    const int cols = m0 + lane < p.M ? p.N - n : 0;
+    float local = 0.f;
+#pragma unroll 1
+    for (int j = 0; j < 32; j += 8) {
+        float cv[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (has_c && j + i < cols) cv[i] = Cp[i * ldc];
+        }
+        const float4 x = *(const float4*)(S + xpose_at(lane, j >> 2)),
+                     y = *(const float4*)(S + xpose_at(lane, (j >> 2) + 1));
+        const float w[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (j + i >= cols) break;
+            float v = alpha * w[i];
+            if (has_c) v = fmaf(beta, cv[i], v);
+            if (md == j + i) v += gamma;
+            Dp[i * ldd] = v;
+            if constexpr (SPLIT) {
+                float h, l;
+                split_tf32(v, h, l);
+                Hp[i * ldd] = h;
+                Lp[i * ldd] = l;
+            }
+            if (has_dot) local += v * v;
+        }
+        Dp += 8 * ldd;
+        if constexpr (SPLIT) {
+            Hp += 8 * ldd;
+            Lp += 8 * ldd;
+        }
+        Cp += has_c ? 8 * ldc : 0;
+    }
+    return local;
+}
+
+// The parked block by the four-element form.
+__device__ __forceinline__ float epi_block32_parked(const EpiParams<float>& p, int m0, int n, float* S,
+                                                 int lane) {
+    const bool split = p.Dhi != nullptr;
+    if (p.trans_block > 0)
+        return split ? epi_block32_trans_vec<true>(p, m0, n, S, lane)
+                     : epi_block32_trans_vec<false>(p, m0, n, S, lane);
+    if (p.sym)
+        return split ? epi_block32_vec<true, true>(p, m0, n, S, lane)
+                     : epi_block32_vec<true, false>(p, m0, n, S, lane);
+    return split ? epi_block32_vec<false, true>(p, m0, n, S, lane)
+                 : epi_block32_vec<false, false>(p, m0, n, S, lane);
+}
+
+// The masked element-wise form of a block in the 33-word layout.
+__device__ __forceinline__ float epi_block32_masked(const EpiParams<float>& p, int m0, int n, bool diag,
+                                                 float* S, int lane) {
+    const bool split = p.Dhi != nullptr;
+    if (p.trans_block > 0)
+        return split ? epi_block32_trans<true>(p, m0, n, S, lane)
+                     : epi_block32_trans<false>(p, m0, n, S, lane);
+    if (p.sym)
+        return split ? epi_block32_plain<true, true>(p, m0, n, diag, S, lane)
+                     : epi_block32_plain<true, false>(p, m0, n, diag, S, lane);
+    return split ? epi_block32_plain<false, true>(p, m0, n, diag, S, lane)
+                 : epi_block32_plain<false, false>(p, m0, n, diag, S, lane);
+}
+
 // Applies the epilogue (alpha, beta C, gamma I, transposed placement, TF32 split copies,
 // symmetric mirror, Frobenius dot; the same arithmetic as epi_apply and epi_apply_sym) to
 // the block of an output tile with rows m0 .. m0 + 31 and columns n .. n + 31. Lane l holds
@@ -186,21 +396,31 @@ __device__ __forceinline__ float epi_block32_trans(const EpiParams<float>& p, in
 __device__ __forceinline__ float epi_block32(const EpiParams<float>& p, int m0, int n,
                                              bool diag, const float (&a)[32], float* S,
                                              int lane) {
-    float local = 0.f;
-    xpose_in(a, S, lane);
+    // outside the matrix, or below the diagonal of a symmetric result
+    if (m0 >= p.M || n >= p.N || (diag && n + 31 < m0)) return 0.f;
+    bool vec = !(diag && n < m0 + 32) && !(p.dot && p.E);
     if (p.trans_block > 0) {
-        local = p.Dhi ? epi_block32_trans<true>(p, m0, n, S, lane)
-                      : epi_block32_trans<false>(p, m0, n, S, lane);
-        __syncwarp();
-        return local;
+        const int last = m0 + 31 < p.M ? m0 + 31 : p.M - 1;
+        vec = vec && m0 / p.trans_block == last / p.trans_block;
+    } else {
+        vec = vec && (n + 32 <= p.N || (p.N & 3) == 0);
+        const uintptr_t al = (uintptr_t)p.D | (uintptr_t)p.Dhi | (uintptr_t)p.Dlo |
+                             (p.beta != 0.f ? (uintptr_t)p.C : 0);
+        const int lds = p.ldd | (p.beta != 0.f ? p.ldc : 0);
+        vec = vec && (al & 15) == 0 && (lds & 3) == 0;
     }
-    const bool split = p.Dhi != nullptr;
-    if (p.sym)
-        local = split ? epi_block32_plain<true, true>(p, m0, n, diag, S, lane)
-                      : epi_block32_plain<true, false>(p, m0, n, diag, S, lane);
-    else
-        local = split ? epi_block32_plain<false, true>(p, m0, n, diag, S, lane)
-                      : epi_block32_plain<false, false>(p, m0, n, diag, S, lane);
+    float local;
+    if (vec) {
+#pragma unroll
+        for (int j = 0; j < 32; j += 4)
+            *(float4*)(S + xpose_at(lane, j >> 2)) =
+                make_float4(a[j], a[j + 1], a[j + 2], a[j + 3]);
+        __syncwarp();
+        local = epi_block32_parked(p, m0, n, S, lane);
+    } else {
+        xpose_in(a, S, lane);
+        local = epi_block32_masked(p, m0, n, diag, S, lane);
+    }
     __syncwarp();   // the buffer is reused by the next block
     return local;
 }
