@@ -1647,7 +1647,8 @@ cdmpt_status Solver<T>::reserve_orders() {
 // the deviation-form image of the paper's C^(m) and B^(m) terms. Each order is
 // solved in correction form d (I + W_k) = -sum_j Z^(q-j)_{k+1} A^(j)_k -
 // 2 Z^(q)_k W_k, Z^(q)_{k+1} = sym(2 Z^(q)_k + d), lower orders first, all with
-// the same step matrix. Start: Z^(1)_0 = -s2 (H1 - mu1 I), Z^(q)_0 = s2 mu^(q) I
+// the same step matrix, whose inverse I - Z_{k+1} Z_k / 2 comes from the trajectory: one
+// product per order (and one symmetric one per step) in place of a CG solve. Start: Z^(1)_0 = -s2 (H1 - mu1 I), Z^(q)_0 = s2 mu^(q) I
 // for q >= 2 (minus s2 H^(q) where given); with the Fermi-Dirac-exact start these are the
 // Y^(q) of tanh_taylor. Only the current and next iterate of each order are kept.
 template <typename T>
@@ -1681,6 +1682,16 @@ cdmpt_status Solver<T>::orders(Context& cx, const double* H1d, const double* H2d
     }
     if (fdx_) CDMPT_TRY(tanh_taylor(cx, m));
     int hint[3] = {1, 1, 1};
+    const bool closed = closed_tangent(o);
+    oz_step_[0] = oz_step_[1] = -1;
+    if (closed && m == 1) {   // first order alone: the tangent of each step
+        for (int k = 0; k < n; ++k) {
+            CDMPT_TRY(need(cx, k));
+            CDMPT_TRY(tangent_step(cx, k, 1, cur(1), nxt(1), acc));
+            cur_[0] ^= 1;
+        }
+        return CDMPT_OK;
+    }
     for (int k = 0; k < n; ++k) {
         CDMPT_TRY(need(cx, k));
         // A^(q)_k from the step-k iterates: S = Z^(q) Z + sum_{1 <= i < q-i} Z^(q-i) Z^(i)
@@ -1712,6 +1723,11 @@ cdmpt_status Solver<T>::orders(Context& cx, const double* H1d, const double* H2d
                                acc));
             }
         }
+        if (closed) {   // -B_k / 2, so that A_k^-1 = I - B_k / 2 takes one product per order
+            CDMPT_TRY(step_product(cx, k, acc));
+            CDMPT_TRY(Ew<T>::axpby(A1_.x, S_.x, blk_, -0.5, 0.0, nullptr, cx.stream, A1_.hi,
+                                   A1_.lo));
+        }
         for (int q = 1; q <= m; ++q) {
             // RHS = -sum_{j=1..q} Z^(q-j)_{k+1} A^(j)_k = -sum_j (A^(j)_k Z^(q-j)_{k+1})^T
             for (int j = 1; j <= q; ++j) {
@@ -1732,7 +1748,22 @@ cdmpt_status Solver<T>::orders(Context& cx, const double* H1d, const double* H2d
                 ep.beta = 1.0;
                 ep.C = RHS_.x;
                 ep.ldc = ld;
+                if (closed) {
+                    ep.Dhi = RHS_.hi;
+                    ep.Dlo = RHS_.lo;
+                }
                 CDMPT_TRY(gemm(cx, N, N, N, cur(q).op(), W_[k].op(), RHS_.x, ep, nullptr, acc));
+            }
+            if (closed) {   // d = RHS A_k^-1
+                Epilogue<T> ep;
+                ep.beta = 1.0;
+                ep.C = RHS_.x;
+                ep.ldc = ld;
+                Buf<T>& Zq = nxt(q);
+                CDMPT_TRY(gemm(cx, N, N, N, RHS_.op(), A1_.op(), Zq.x, ep, nullptr, acc));
+                CDMPT_TRY(Ew<T>::axpby(Zq.x, cur(q).x, blk_, 2.0, 1.0, nullptr, cx.stream));
+                CDMPT_TRY(Ew<T>::symmetrize(Zq.x, N, ld, 1, cx.stream, Zq.hi, Zq.lo));
+                continue;
             }
             CgArgs a;
             a.W = &W_[k];
@@ -1799,6 +1830,10 @@ cdmpt_status Solver<T>::higher(Context& cx, const double* H1, int D, int m, cons
             CDMPT_CUDA_TRY(cudaMemsetAsync(sc_ + S_TRQ + 1, 0, sizeof(double), cx.stream));
             CDMPT_TRY(Ew<T>::trace(Zq.x, N, ld, 1, sc_ + S_TRQ + 1, cx.stream));
             CDMPT_TRY(read_scalars(cx, sc_, S_NSLOTS));
+            if (sizeof(T) == 4 && closed_tangent(o) && !std::isfinite(cx.pinned[S_TRQ + 1])) {
+                set_error("the response met a non-finite value: no solution of its linear systems");
+                return CDMPT_ERR_CG_MAXITER;
+            }
             const double muq = gc ? 0.0 : -0.5 * cx.pinned[S_TRQ + 1] / trQ;
             if (q < m) {
                 mus[q - 1] = muq;
@@ -1901,32 +1936,65 @@ cdmpt_status Solver<T>::logdet(Context& cx, const Buf<T>& M, double a, double b,
     Buf<T>& Y2 = zo_[0][1];
     Buf<T>* Pw = &zo_[1][0];
     Buf<T>* Pn = &zo_[1][1];
-    // Y (A + c I) = A - c I with A = a I + b M: operator X -> (a + c) X + b X M
-    CDMPT_TRY(Ew<T>::axpby(RHS_.x, M.x, blk_, b, 0.0, nullptr, cx.stream));
-    CDMPT_TRY(Ew<T>::add_diag(RHS_.x, N, ld, 1, a - c, cx.stream));
-    CgArgs g;
-    g.W = &M;
-    g.s = a + c;
-    g.t = b;
-    g.rhs = RHS_.x;
-    g.rows = N;
-    g.tol = o.cg_tol;
-    g.maxit = o.cg_maxit;
-    g.init_engine = g.iter_engine = acc;
-    g.hint = 4;
-    int it = 0;
-    CDMPT_TRY(cg(cx, Y.x, g, &it, nullptr));
-    CDMPT_TRY(Ew<T>::symmetrize(Y.x, N, ld, 1, cx.stream, Y.hi, Y.lo));
-    auto trace_of = [&](const Buf<T>& B, double* v) -> cdmpt_status {
-        CDMPT_CUDA_TRY(cudaMemsetAsync(sc_ + S_FE, 0, sizeof(double), cx.stream));
-        CDMPT_TRY(Ew<T>::trace(B.x, N, ld, 1, sc_ + S_FE, cx.stream));
+    // Y (A + c I) = A - c I with A = a I + b M: operator X -> (a + c) X + b X M. With b = +-1 the
+    // spectrum of b M is known, so (A + c I)^-1 is a polynomial in M (InversePoly) and Y one more
+    // product, all on upper-triangle tiles; Y keeps the relative accuracy of the small A - c I.
+    InversePoly p;
+    if (!(screen_tau_ > 0.f) && std::fabs(b) == 1.0 &&
+        p.fit(a + c, lo - a, hi - a, 0.5 * o.cg_tol,
+              std::min(o.cg_maxit, sizeof(T) == 8 ? 20 : 16))) {
+        for (int j = 1; j <= p.degree(); j += 2) p.a[j] *= b;   // (b M - c)^j, b = +-1
+        p.c *= b;
+        const Buf<T>* E = &P_;
+        if (p.degree() == 1) {
+            CDMPT_TRY(Ew<T>::axpby(P_.x, M.x, blk_, p.a[1], 0.0, nullptr, cx.stream, P_.hi, P_.lo));
+            CDMPT_TRY(Ew<T>::add_diag(P_.x, N, ld, 1, p.a[0] - p.a[1] * p.c, cx.stream, P_.hi,
+                                      P_.lo));
+        } else {
+            CDMPT_TRY(poly_eval(cx, M, p, 0.0, acc, &E));
+        }
+        Buf<T>& L = E == &A1_ ? RHS_ : A1_;   // A - c I
+        CDMPT_TRY(Ew<T>::axpby(L.x, M.x, blk_, b, 0.0, nullptr, cx.stream, L.hi, L.lo));
+        CDMPT_TRY(Ew<T>::add_diag(L.x, N, ld, 1, a - c, cx.stream, L.hi, L.lo));
+        Epilogue<T> ep;
+        ep.Dhi = Y.hi;
+        ep.Dlo = Y.lo;
+        ep.sym = true;
+        CDMPT_TRY(gemm(cx, N, N, N, L.op(), E->op(), Y.x, ep, nullptr, acc));
+        if (engine_of(cx, acc) == CDMPT_GEMM_SIMT)   // full tiles, not mirrored
+            CDMPT_TRY(Ew<T>::symmetrize(Y.x, N, ld, 1, cx.stream, Y.hi, Y.lo));
+    } else {
+        CDMPT_TRY(Ew<T>::axpby(RHS_.x, M.x, blk_, b, 0.0, nullptr, cx.stream));
+        CDMPT_TRY(Ew<T>::add_diag(RHS_.x, N, ld, 1, a - c, cx.stream));
+        CgArgs g;
+        g.W = &M;
+        g.s = a + c;
+        g.t = b;
+        g.rhs = RHS_.x;
+        g.rows = N;
+        g.tol = o.cg_tol;
+        g.maxit = o.cg_maxit;
+        g.init_engine = g.iter_engine = acc;
+        g.hint = 4;
+        int it = 0;
+        CDMPT_TRY(cg(cx, Y.x, g, &it, nullptr));
+        CDMPT_TRY(Ew<T>::symmetrize(Y.x, N, ld, 1, cx.stream, Y.hi, Y.lo));
+    }
+    // traces of the terms into slots of their own, read back once (every 16 terms)
+    constexpr int kTerms = S_NSLOTS - S_FE;
+    double sum = 0.0;
+    int first = 0;
+    CDMPT_CUDA_TRY(cudaMemsetAsync(sc_ + S_FE, 0, kTerms * sizeof(double), cx.stream));
+    auto trace_of = [&](const Buf<T>& B, int j) -> cdmpt_status {   // term j of sum / (2 j + 1)
+        CDMPT_TRY(Ew<T>::trace(B.x, N, ld, 1, sc_ + S_FE + (j - first), cx.stream));
+        if (j < J && j - first + 1 < kTerms) return CDMPT_OK;
         CDMPT_TRY(read_scalars(cx, sc_, S_NSLOTS));
-        *v = cx.pinned[S_FE];
+        for (int i = first; i <= j; ++i) sum += cx.pinned[S_FE + (i - first)] / (2 * i + 1);
+        first = j + 1;
+        CDMPT_CUDA_TRY(cudaMemsetAsync(sc_ + S_FE, 0, kTerms * sizeof(double), cx.stream));
         return CDMPT_OK;
     };
-    double sum = 0.0, t = 0.0;
-    CDMPT_TRY(trace_of(Y, &t));
-    sum = t;
+    CDMPT_TRY(trace_of(Y, 0));
     if (J > 0) {
         Epilogue<T> ep;   // Y^2 (symmetric)
         ep.Dhi = Y2.hi;
@@ -1939,9 +2007,9 @@ cdmpt_status Solver<T>::logdet(Context& cx, const Buf<T>& M, double a, double b,
         Epilogue<T> ep;
         ep.Dhi = Pn->hi;
         ep.Dlo = Pn->lo;
+        ep.sym = true;   // powers of one symmetric matrix
         CDMPT_TRY(gemm(cx, N, N, N, odd->op(), Y2.op(), Pn->x, ep, nullptr, acc));
-        CDMPT_TRY(trace_of(*Pn, &t));
-        sum += t / (2 * j + 1);
+        CDMPT_TRY(trace_of(*Pn, j));
         odd = Pn;
         std::swap(Pw, Pn);
     }
