@@ -491,6 +491,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             float* const Dlp = p.Dl;
             float* const Dth = p.Dthi;
             float* const Dtl = p.Dtlo;
+            const bool vec =
+                ((ldc | ldd) & 3) == 0 &&
+                (((uintptr_t)c1h | (uintptr_t)c1l | (uintptr_t)c2h | (uintptr_t)c2l |
+                  (uintptr_t)Dp | (uintptr_t)Dlp | (uintptr_t)Dth | (uintptr_t)Dtl) &
+                 15) == 0;
 #pragma unroll 1
             for (int c0 = 0; c0 < CW; c0 += 8) {
                 uint32_t r[ND][8];
@@ -499,76 +504,114 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                 tmem_ld_wait();
                 if (row_ok) {
                     const size_t rowc = (size_t)m * ldc, rowd = (size_t)m * ldd;
-                    // the chunk's loads first (column exponents and C terms), then its
-                    // arithmetic and stores: one memory latency per chunk, not per element
+                    const int n8 = n0 + c0;
+                    // A lane's eight columns are 32 bytes of its row: two 16-byte accesses per
+                    // array where all of them are taken, against eight that each touch a sector
+                    // of every row (32 rows per warp: eight times the L2 transactions)
+                    const bool full = vec && n8 + 8 <= PN && (!sym || n8 >= m);
                     int eyv[8];
                     float ch1[8], cl1[8], ch2[8], cl2[8];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int n = n0 + c0 + j;
-                        const bool ok = n < PN && !(sym && n < m);
-                        eyv[j] = ok ? ey[n] : 0;
-                        ch1[j] = (ok && c1h) ? c1h[rowc + n] : 0.f;
-                        cl1[j] = (ok && c1l) ? c1l[rowc + n] : 0.f;
-                        ch2[j] = (ok && c2h) ? c2h[rowc + n] : 0.f;
-                        cl2[j] = (ok && c2l) ? c2l[rowc + n] : 0.f;
-                    }
-                    float local = 0.f;
+                    for (int j = 0; j < 8; ++j) eyv[j] = n8 + j < PN ? ey[n8 + j] : 0;
+                    auto load8 = [&](const float* c, float (&v)[8]) {
+                        if (c && full) {
+                            const float4 x = *(const float4*)(c + rowc + n8);
+                            const float4 y = *(const float4*)(c + rowc + n8 + 4);
+                            v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+                            v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+                        } else {
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int n = n0 + c0 + j;
-                        if (n < PN && !(sym && n < m)) {
-                            // exact integer part of the exact groups, then the float tail of the
-                            // whole-K groups, in units of the last exact group's weight
-                            long long I = 0;
-#pragma unroll
-                            for (int g = 0; g < NX; ++g) I = I * 256 + (long long)(int)r[g][j];
-                            float vh = (float)I;
-                            float vl = (float)(I - (long long)vh);
-                            vl = __fadd_rn(vl, __fadd_rn(__uint_as_float(r[NX][j]) * (1.f / 256.f),
-                                                         __uint_as_float(r[NX + 1][j]) * (1.f / 65536.f)));
-                            const int sh = ex + eyv[j] - 14 - 8 * (NX - 1);
-                            vh = scale2(vh, sh);
-                            vl = scale2(vl, sh);
-                            // D = alpha X Y^T + b1 C1 + b2 C2 + gamma I in double-float
-                            float dh = __fmul_rn(alpha, vh), dl = __fmul_rn(alpha, vl);
-                            if (c1h) {
-                                const float ch = __fmul_rn(b1, ch1[j]);
-                                const float cl = c1l ? __fmul_rn(b1, cl1[j]) : 0.f;
-                                dd::add(dh, dl, ch, cl, dh, dl);
+                            for (int j = 0; j < 8; ++j) {
+                                const int n = n8 + j;
+                                v[j] = (c && n < PN && !(sym && n < m)) ? c[rowc + n] : 0.f;
                             }
-                            if (c2h) {
-                                const float ch = __fmul_rn(b2, ch2[j]);
-                                const float cl = c2l ? __fmul_rn(b2, cl2[j]) : 0.f;
-                                dd::add(dh, dl, ch, cl, dh, dl);
-                            }
-                            if (gamma != 0.f && n == m) dd::add1(dh, dl, gamma, dh, dl);
-                            float o, ol;
-                            dd::fast_two_sum(dh, dl, o, ol);
-                            // symmetric result: the mirror (n, m) too (the lanes hold
-                            // consecutive rows m, so these stores coalesce)
-                            const bool mir = sym && n > m;
-                            const size_t mirror = (size_t)n * ldd + m;
-                            Dp[rowd + n] = o;
-                            if (mir) Dp[mirror] = o;
-                            if (Dlp) {
-                                Dlp[rowd + n] = ol;
-                                if (mir) Dlp[mirror] = ol;
-                            }
-                            if (Dth) {
-                                float th, tl;
-                                dd::tf32_split(o, th, tl);
-                                Dth[rowd + n] = th;
-                                if (mir) Dth[mirror] = th;
-                                if (Dtl) {
-                                    Dtl[rowd + n] = tl;
-                                    if (mir) Dtl[mirror] = tl;
-                                }
-                            }
-                            local = __fmaf_rn(mir ? 2.f * o : o, o, local);
                         }
+                    };
+                    load8(c1h, ch1);
+                    load8(c1l, cl1);
+                    load8(c2h, ch2);
+                    load8(c2l, cl2);
+                    float o[8], ol[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        // exact integer part of the exact groups, then the float tail of the
+                        // whole-K groups, in units of the last exact group's weight
+                        long long I = 0;
+#pragma unroll
+                        for (int g = 0; g < NX; ++g) I = I * 256 + (long long)(int)r[g][j];
+                        float vh = (float)I;
+                        float vl = (float)(I - (long long)vh);
+                        vl = __fadd_rn(vl, __fadd_rn(__uint_as_float(r[NX][j]) * (1.f / 256.f),
+                                                     __uint_as_float(r[NX + 1][j]) * (1.f / 65536.f)));
+                        const int sh = ex + eyv[j] - 14 - 8 * (NX - 1);
+                        o[j] = __fmul_rn(alpha, scale2(vh, sh));
+                        ol[j] = __fmul_rn(alpha, scale2(vl, sh));
                     }
-                    dsum += (double)local;
+                    // D = alpha X Y^T + b1 C1 + b2 C2 + gamma I in double-float
+                    if (c1h) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            dd::add(o[j], ol[j], __fmul_rn(b1, ch1[j]), __fmul_rn(b1, cl1[j]), o[j],
+                                    ol[j]);
+                    }
+                    if (c2h) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            dd::add(o[j], ol[j], __fmul_rn(b2, ch2[j]), __fmul_rn(b2, cl2[j]), o[j],
+                                    ol[j]);
+                    }
+                    if (gamma != 0.f) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            if (n8 + j == m) dd::add1(o[j], ol[j], gamma, o[j], ol[j]);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float dh = o[j], dl = ol[j];
+                        dd::fast_two_sum(dh, dl, o[j], ol[j]);
+                    }
+                    // the rows, and for a symmetric result the mirror (n, m) (the lanes hold
+                    // consecutive rows m, so those stores coalesce)
+                    auto store8 = [&](float* d, const float (&v)[8]) {
+                        if (full) {
+                            *(float4*)(d + rowd + n8) = make_float4(v[0], v[1], v[2], v[3]);
+                            *(float4*)(d + rowd + n8 + 4) = make_float4(v[4], v[5], v[6], v[7]);
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) {
+                                const int n = n8 + j;
+                                if (n < PN && !(sym && n < m)) d[rowd + n] = v[j];
+                            }
+                        }
+                        if (sym) {
+                            float* q = d + (size_t)n8 * ldd + m;
+#pragma unroll
+                            for (int j = 0; j < 8; ++j, q += ldd)
+                                if (n8 + j < PN && n8 + j > m) *q = v[j];
+                        }
+                    };
+                    store8(Dp, o);
+                    if (Dlp) store8(Dlp, ol);
+                    if (p.dot) {
+                        float local = 0.f;
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const int n = n8 + j;
+                            const float w = (sym && n > m) ? 2.f * o[j] : o[j];
+                            if (n < PN && !(sym && n < m)) local = __fmaf_rn(w, o[j], local);
+                        }
+                        dsum += (double)local;
+                    }
+                    if (Dth) {
+                        float th[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const float v = o[j];
+                            dd::tf32_split(v, th[j], ol[j]);
+                        }
+                        store8(Dth, th);
+                        if (Dtl) store8(Dtl, ol);
+                    }
                 }
             }
             tc_fence_before();
@@ -598,44 +641,108 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     }
 }
 
-// One warp per row: the row's power of two and the ND BF16 digits of every element.
+// round(x 2^sh') of a float's bits to nearest even, where sh' takes the row's largest biased
+// exponent emax >= 1 to the top of BITS bits (x 2^(BITS - e), e = emax - 126).
+template <int BITS>
+__device__ __forceinline__ long long oz_fixed(uint32_t b, int emax) {
+    const int eb = (int)(b >> 23) & 0xff;
+    unsigned long long M = b & 0x7fffffu;
+    if (eb) M |= 1u << 23;
+    const int sh = (eb ? eb : 1) - emax + BITS - 24;
+    unsigned long long t;
+    if (sh >= 0) {
+        t = M << sh;
+    } else if (sh > -26) {
+        const unsigned long long half = 1ull << (-sh - 1), rest = M & (2ull * half - 1ull);
+        t = M >> -sh;
+        t += (rest > half || (rest == half && (t & 1ull))) ? 1ull : 0ull;
+    } else {
+        t = 0ull;
+    }
+    return (b >> 31) ? -(long long)t : (long long)t;
+}
+
+// One block per row: the row's power of two and the ND BF16 digits of every element. Bound by
+// memory (8 bytes in, 2 ND out, per element); four columns per thread, so that a warp writes
+// 256 bytes of each digit array at a time, and integer operations on the float's bits instead
+// of 64-bit conversions (one warp per row with two-byte stores took 117 us at N = 4096, 44 us
+// at the copy rate).
+constexpr int OZ_SLICE_THREADS = 128;
 template <int ND>
-__global__ void k_oz_slice(const float* __restrict__ xh, const float* __restrict__ xl, int rows,
-                           int cols, int ld, OzOperand out) {
+__global__ void __launch_bounds__(OZ_SLICE_THREADS)
+    k_oz_slice(const float* __restrict__ xh, const float* __restrict__ xl, int rows, int cols,
+               int ld, OzOperand out) {
     constexpr int BITS = 8 * ND - 1;
-    const int lane = threadIdx.x & 31;
-    const int wpb = blockDim.x >> 5;
-    for (int r = blockIdx.x * wpb + (threadIdx.x >> 5); r < rows; r += gridDim.x * wpb) {
+    __shared__ int wmax[OZ_SLICE_THREADS / 32];
+    const bool vec = (((uintptr_t)xh | (uintptr_t)xl) & 15) == 0;   // ld is a multiple of 8
+    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
         const float* hr = xh + (size_t)r * ld;
         const float* lr = xl ? xl + (size_t)r * ld : nullptr;
-        float mx = 0.f;
-        for (int j = lane; j < cols; j += 32) mx = fmaxf(mx, fabsf(hr[j]));
+        auto load4 = [&](const float* x, int j, uint32_t (&b)[4]) {
+            if (vec && j + 4 <= cols) {
+                const uint4 u = *(const uint4*)(x + j);
+                b[0] = u.x;
+                b[1] = u.y;
+                b[2] = u.z;
+                b[3] = u.w;
+            } else {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        int e = 0;
-        if (mx > 0.f) (void)frexpf(mx, &e);   // mx = m 2^e, m in [0.5, 1): |x| 2^-e < 1
-        if (lane == 0) out.e[r] = e;
+                for (int i = 0; i < 4; ++i) b[i] = j + i < cols ? __float_as_uint(x[j + i]) : 0u;
+            }
+        };
+        int emax = 0;
+        bool any = false;
+        for (int j = threadIdx.x * 4; j < cols; j += OZ_SLICE_THREADS * 4) {
+            uint32_t b[4];
+            load4(hr, j, b);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                emax = max(emax, (int)(b[i] >> 23) & 0xff);
+                any |= (b[i] << 1) != 0u;
+            }
+        }
+        // a row of subnormal numbers counts as exponent 1, an all-zero row as none
+        emax = any ? max(emax, 1) : 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+        if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = emax;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < OZ_SLICE_THREADS / 32; ++w) emax = max(emax, wmax[w]);
+        __syncthreads();
+        if (threadIdx.x == 0) out.e[r] = emax ? emax - 126 : 0;
         const size_t off = (size_t)r * ld;
-        for (int j = lane; j < ld; j += 32) {
-            int dg[ND];
+        for (int j = threadIdx.x * 4; j < ld; j += OZ_SLICE_THREADS * 4) {
+            uint32_t h[4], l[4] = {0u, 0u, 0u, 0u};
+            load4(hr, j, h);
+            if (lr) load4(lr, j, l);
+            uint32_t dg[ND][2];
 #pragma unroll
-            for (int d = 0; d < ND; ++d) dg[d] = 0;
-            if (j < cols && mx > 0.f) {
-                // T = round((xh + xl) 2^(BITS - e)), |T| <= 2^BITS; digits by round-to-nearest
-                long long T = __float2ll_rn(scale2(hr[j], BITS - e));
-                if (lr) T += __float2ll_rn(scale2(lr[j], BITS - e));
+            for (int i = 0; i < 4; ++i) {
+                long long T = 0;
+                if (emax) T = oz_fixed<BITS>(h[i], emax) + oz_fixed<BITS>(l[i], emax);
 #pragma unroll
-                for (int d = 0; d < ND - 1; ++d) {
+                for (int d = 0; d < ND; ++d) {
                     const int sh = 8 * (ND - 1 - d);
-                    const long long a = (T + (1ll << (sh - 1))) >> sh;
-                    dg[d] = (int)a;
-                    T -= a << sh;
+                    int v;
+                    if (d < ND - 1) {
+                        const long long a = (T + (1ll << (sh - 1))) >> sh;
+                        v = (int)a;
+                        T -= a << sh;
+                    } else {
+                        v = (int)T;
+                    }
+                    // |v| <= 128: the upper half of its FP32 form is its BF16 form, exactly
+                    const uint32_t f = __float_as_uint((float)v) >> 16;
+                    if ((i & 1) == 0)
+                        dg[d][i >> 1] = f;
+                    else
+                        dg[d][i >> 1] |= f << 16;
                 }
-                dg[ND - 1] = (int)T;
             }
 #pragma unroll
             for (int d = 0; d < ND; ++d)
-                ((__nv_bfloat16*)out.s[d])[off + j] = __float2bfloat16_rn((float)dg[d]);
+                *(uint2*)((__nv_bfloat16*)out.s[d] + off + j) = make_uint2(dg[d][0], dg[d][1]);
         }
     }
 }
@@ -735,13 +842,11 @@ cdmpt_status oz_slice(const float* xh, const float* xl, int rows, int cols, int 
         set_error("Ozaki slicing: 4 or 5 digits, cols <= 32768, cols <= ld, ld a multiple of 8");
         return CDMPT_ERR_ARG;
     }
-    const int wpb = 8;
-    int grid = (rows + wpb - 1) / wpb;
-    if (grid > 152 * 16) grid = 152 * 16;
+    const int grid = rows < 152 * 16 ? rows : 152 * 16;
     if (nd == 5)
-        k_oz_slice<5><<<grid, 32 * wpb, 0, s>>>(xh, xl, rows, cols, ld, out);
+        k_oz_slice<5><<<grid, OZ_SLICE_THREADS, 0, s>>>(xh, xl, rows, cols, ld, out);
     else
-        k_oz_slice<4><<<grid, 32 * wpb, 0, s>>>(xh, xl, rows, cols, ld, out);
+        k_oz_slice<4><<<grid, OZ_SLICE_THREADS, 0, s>>>(xh, xl, rows, cols, ld, out);
     count_launch();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
