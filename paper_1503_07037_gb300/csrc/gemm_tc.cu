@@ -240,7 +240,8 @@ __global__ void __launch_bounds__(tc_threads(KCH), 1)
     volatile int* abort_flag = (volatile int*)(tmem_holder + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // symmetric results (p.sym, square tiles) enumerate the upper-triangular tiles only
+    // symmetric results (p.sym; 128 or 64 columns) enumerate the tiles that meet the upper
+    // triangle only
     const int2* tcache = (const int2*)(smem + STAGES * C::STAGE_BYTES + 256);
     auto tile = [&](int t) {
         const int li = (t - (int)blockIdx.x) / (int)gridDim.x;
@@ -254,6 +255,15 @@ __global__ void __launch_bounds__(tc_threads(KCH), 1)
             r.m0 = mi * BM;
             r.n0 = ni * BN;
             r.diag = mi == ni;
+        } else if (2 * BN == BM && r.pr->p.sym) {
+            // column tile ni has ni / 2 + 1 row tiles, a (a + 1) stand before ni = 2 a
+            int a = (int)((sqrtf(4.f * (float)lt + 1.f) - 1.f) * 0.5f);
+            while (a * (a + 1) > lt) --a;
+            while ((a + 1) * (a + 2) <= lt) ++a;
+            const int rem = lt - a * (a + 1), ni = 2 * a + rem / (a + 1), mi = rem % (a + 1);
+            r.m0 = mi * BM;
+            r.n0 = ni * BN;
+            r.diag = mi == ni / 2;
         } else {
             r.n0 = (lt / r.pr->num_mt) * BN;
         }
@@ -650,6 +660,16 @@ cdmpt_status set_smem_attr() {
     return CDMPT_OK;
 }
 
+// Output tiles of bm x bn (bn = bm or bm / 2 for a symmetric result)
+int tile_count(int bm, int bn, int M, int N, bool sym) {
+    const int mt = (M + bm - 1) / bm, nt = (N + bn - 1) / bn;
+    if (!sym) return mt * nt;
+    const int per = bm / bn;
+    int t = 0;
+    for (int j = 0; j < nt; ++j) t += j / per + 1;
+    return t;
+}
+
 template <int BN, int STAGES, int PASSES, int KCH, bool SCREEN = false>
 cdmpt_status launch(int M, int N, int K, const float* X, const float* Xl, int ldx, const float* Y,
                     const float* Yl, int ldy, const EpiParams<float>& p, const double* skip,
@@ -681,10 +701,10 @@ cdmpt_status launch(int M, int N, int K, const float* X, const float* Xl, int ld
     pr.nnt = SCREEN ? (N + BM - 1) / BM : 0;
     pr.nmw = SCREEN ? sc->nmw : 0;
     pr.counts = SCREEN ? sc->counts : nullptr;
-    // symmetric results need square tiles: upper-triangular tiles only
-    const bool sym = p.sym && BN == BM && M == N;
+    // symmetric results: the tiles that meet the upper triangle only
+    const bool sym = p.sym && (BN == BM || 2 * BN == BM) && M == N;
     pr.p.sym = sym ? 1 : 0;
-    const int tiles = sym ? pr.num_mt * (pr.num_mt + 1) / 2 : pr.num_mt * ((N + BN - 1) / BN);
+    const int tiles = tile_count(BM, BN, M, N, sym);
     const int grid = tiles < sm_count() ? tiles : sm_count();
     k_gemm_tc<BN, STAGES, PASSES, KCH, false, SCREEN><<<grid, tc_threads(KCH), C::SMEM, s>>>(
         mx, my, mxl, myl, pr, nullptr, 1, tiles, device_error_word());
@@ -697,31 +717,37 @@ cdmpt_status launch(int M, int N, int K, const float* X, const float* Xl, int ld
     return CDMPT_OK;
 }
 
-// Kernel family for single (non-grouped) products with more than 128 rows: 128 x 128 tiles on
-// one SM, or 256 x 256 tiles on an SM pair (cta_group::2; for split TF32 the wide kernel
-// k_gemm_split2sm). Both take about the same time per tile and k (split 25 ns, one-pass 9 ns),
-// the pair's tile having twice the work per SM, and a fixed part that the larger tile's
-// epilogue lengthens (in units of k: split 330 and 590; one-pass 700 and 1000). So the small tile
-// wins where its tiles still fit one wave or the pairs' tiles leave SMs idle, and the line is
-// drawn by the waves of either. Measured, split, one SM against two: N = 512 21 and 28 us,
-// 1536 46 and 54, 2048 107 and 68 (63 and 70 for a symmetric result), 4096 687 and 477.
-// CDMPT_TC_MODE=1sm|2sm forces one family.
-bool use_2sm(bool three, int M, int N, int K, bool sym) {
-    static int v = -2;
-    if (v == -2) {
+// Tiles of single (non-grouped) products: 128 x 64 or 128 x 128 on one SM, or 256 x 256 on an SM
+// pair (cta_group::2; for split TF32 the wide kernel k_gemm_split2sm). In units of the time a
+// 128 x 128 tile takes per k (split 25 ns, one-pass 9 ns), the pair's tile takes the same (twice
+// the work per SM) and the 64-column tile about as much too (its k-loop waits for the same number
+// of copies); each has a fixed part besides, longer for the larger epilogue. So the smaller
+// tiles win where theirs still fit one wave of SMs, and the line is drawn by the waves of each.
+// Measured, split, 64 and 128 columns and the pair: N = 512 19, 23 and 28 us, 1000 31, 35 and 50,
+// 1536 78, 47 and 54, 2048 195, 107 and 68 (symmetric result 105, 64 and 70), 4096 1306, 685
+// and 478.
+// CDMPT_TC_MODE=64|1sm|2sm forces one family.
+enum TileFamily { TILE_64, TILE_128, TILE_PAIR };
+TileFamily tile_family(bool three, int M, int N, int K, bool sym) {
+    static int forced = -2;
+    if (forced == -2) {
         const char* e = getenv("CDMPT_TC_MODE");
-        v = !e ? -1 : (std::strcmp(e, "2sm") == 0 ? 1 : 0);
+        forced = !e ? -1
+                    : std::strcmp(e, "2sm") == 0 ? TILE_PAIR
+                                                 : std::strcmp(e, "64") == 0 ? TILE_64 : TILE_128;
     }
-    if (v >= 0) return v == 1;
-    auto waves = [&](int t, int slots) {
-        const long long mt = (M + t - 1) / t, nt = (N + t - 1) / t;
-        const long long tiles = sym ? mt * (mt + 1) / 2 : mt * nt;
-        return (double)((tiles + slots - 1) / slots);
-    };
+    if (forced >= 0) return (TileFamily)(forced == TILE_PAIR && M <= BM ? (int)TILE_128 : forced);
     const int sms = sm_count();
-    const double one = waves(BM, sms) * (K + (three ? 330 : 700));
-    const double two = waves(2 * BM, std::max(1, sms / 2)) * (K + (three ? 590 : 1000));
-    return two < one;
+    auto cost = [&](int bm, int bn, int slots, double per_k, double fixed) {
+        const int t = tile_count(bm, bn, M, N, sym);
+        return (double)((t + slots - 1) / slots) * (per_k * K + fixed);
+    };
+    const double c64 = cost(BM, 64, sms, 1.0, three ? 180 : 400);
+    const double c128 = cost(BM, BM, sms, 1.0, three ? 330 : 700);
+    const double pair = M > BM ? cost(2 * BM, 2 * BM, std::max(1, sms / 2), 1.0, three ? 590 : 1000)
+                               : c128;
+    if (pair < c128 && pair < c64) return TILE_PAIR;
+    return c64 < c128 ? TILE_64 : TILE_128;
 }
 
 template <int BN, int STAGES, int PASSES, int KCH>
@@ -926,10 +952,22 @@ cdmpt_status gemm_tc_f32(int engine, int M, int N, int K, const Operand<float>& 
             default: return launch<128, 3, 3, 2, true>(M, N, K, xh, X.lo, ldx, yh, Y.lo, ldy, p, skip, s, screen);
         }
     }
-    // symmetric results need square tiles: upper triangle only
-    if (M > BM && use_2sm(three, M, N, K, p.sym != 0))
-        return gemm_tc_2sm(three, split_chunk(), M, N, K, xh, three ? X.lo : xh, ldx, yh,
-                           three ? Y.lo : yh, ldy, p, skip, s);
+    switch (tile_family(three, M, N, K, p.sym != 0)) {
+        case TILE_PAIR:
+            return gemm_tc_2sm(three, split_chunk(), M, N, K, xh, three ? X.lo : xh, ldx, yh,
+                               three ? Y.lo : yh, ldy, p, skip, s);
+        case TILE_64:
+            if (!three) return launch<64, 8, 1, 0>(M, N, K, xh, xh, ldx, yh, yh, ldy, p, skip, s);
+            // the chunk of the 128-column kernel, so the same sums
+            switch (split_chunk()) {
+                case 1: return launch<64, 4, 3, 1>(M, N, K, xh, X.lo, ldx, yh, Y.lo, ldy, p, skip, s);
+                case 2: return launch<64, 4, 3, 2>(M, N, K, xh, X.lo, ldx, yh, Y.lo, ldy, p, skip, s);
+                default: break;   // chunks without a 64-column kernel
+            }
+            break;
+        default:
+            break;
+    }
     if (!three) return launch<128, 6, 1, 0>(M, N, K, xh, xh, ldx, yh, yh, ldy, p, skip, s);
     switch (split_chunk()) {
         case 1: return launch<128, 3, 3, 1>(M, N, K, xh, X.lo, ldx, yh, Y.lo, ldy, p, skip, s);
