@@ -296,19 +296,36 @@ __global__ void k_grouped_tiles(const GrpEw* __restrict__ desc, int max_blocks) 
             b[y][x] = (j0 + y < N && i0 + x < N) ? d.p4[base + (size_t)(j0 + y) * ld + i0 + x] : 0.f;
         }
         __syncthreads();
-        auto put_one = [&](int r, int c, float v) {
-            if (r >= N || c >= N) return;
-            const size_t i = base + (size_t)r * ld + c;
-            float h, l;
-            dd::add1(d.p0[i], d.p1[i], v, h, l);
-            d.p0[i] = h;
-            d.p1[i] = l;
-            if (d.p2) split1(h, d.p2, d.p3, i);
+        constexpr int R = TT / 8;   // blockDim.y = 8
+        float h[2][R], l[2][R];
+        auto at = [&](int side, int y) {
+            const int r = (side ? j0 : i0) + y, c = (side ? i0 : j0) + x;
+            return r < N && c < N ? (long long)(base + (size_t)r * ld + c) : -1ll;
         };
-#pragma unroll 4
-        for (int y = threadIdx.y; y < TT; y += blockDim.y) {
-            put_one(i0 + y, j0 + x, 0.5f * (a[y][x] + b[x][y]));
-            if (bi != bj) put_one(j0 + y, i0 + x, 0.5f * (a[x][y] + b[y][x]));
+        // the loads first: a load after a store would wait for it
+#pragma unroll
+        for (int side = 0; side < 2; ++side)
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                const long long i = at(side, threadIdx.y + 8 * q);
+                h[side][q] = i >= 0 ? d.p0[i] : 0.f;
+                l[side][q] = i >= 0 ? d.p1[i] : 0.f;
+            }
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+            if (side && bi == bj) break;
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                const int y = threadIdx.y + 8 * q;
+                const long long i = at(side, y);
+                if (i < 0) continue;
+                const float v = 0.5f * (side ? a[x][y] + b[y][x] : a[y][x] + b[x][y]);
+                float nh, nl;
+                dd::add1(h[side][q], l[side][q], v, nh, nl);
+                d.p0[i] = nh;
+                d.p1[i] = nl;
+                if (d.p2) split1(nh, d.p2, d.p3, i);
+            }
         }
     } else {                   // p0 = p1 + p1^T
         for (int y = threadIdx.y; y < TT; y += blockDim.y) {

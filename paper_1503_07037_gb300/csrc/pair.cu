@@ -176,19 +176,36 @@ __global__ void k_pair_add_sym(float* __restrict__ hi, float* __restrict__ lo,
         b[y][x] = (j0 + y < N && i0 + x < N) ? d[(size_t)(j0 + y) * ld + i0 + x] : 0.f;
     }
     __syncthreads();
-    auto put_one = [&](int r, int c, float s) {
-        if (r >= N || c >= N) return;
-        const size_t i = (size_t)r * ld + c;
-        float h, l;
-        dd::add1(hi[i], lo[i], s, h, l);
-        hi[i] = h;
-        lo[i] = l;
-        put(thi, tlo, i, h);
+    // the eight elements' loads first: a load of hi or lo after a store would wait for it
+    constexpr int R = TT / 8;   // blockDim.y = 8
+    float h[2][R], l[2][R];
+    auto at = [&](int side, int y) {
+        const int r = (side ? j0 : i0) + y, c = (side ? i0 : j0) + x;
+        return r < N && c < N ? (long long)r * ld + c : -1ll;
     };
-#pragma unroll 4
-    for (int y = threadIdx.y; y < TT; y += blockDim.y) {
-        put_one(i0 + y, j0 + x, 0.5f * (a[y][x] + b[x][y]));
-        if (bi != bj) put_one(j0 + y, i0 + x, 0.5f * (a[x][y] + b[y][x]));
+#pragma unroll
+    for (int side = 0; side < 2; ++side)
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            const long long i = at(side, threadIdx.y + 8 * q);
+            h[side][q] = i >= 0 ? hi[i] : 0.f;
+            l[side][q] = i >= 0 ? lo[i] : 0.f;
+        }
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+        if (side && bi == bj) break;
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            const int y = threadIdx.y + 8 * q;
+            const long long i = at(side, y);
+            if (i < 0) continue;
+            const float s = 0.5f * (side ? a[x][y] + b[y][x] : a[y][x] + b[x][y]);
+            float nh, nl;
+            dd::add1(h[side][q], l[side][q], s, nh, nl);
+            hi[i] = nh;
+            lo[i] = nl;
+            put(thi, tlo, i, nh);
+        }
     }
 }
 
