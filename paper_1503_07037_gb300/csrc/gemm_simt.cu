@@ -93,6 +93,10 @@ constexpr int SM_T = 8, SM_KC = 256, SM_G = 4;
 __global__ void __launch_bounds__(SM_G* SM_T* SM_T) k_gemm_small_f64(
     const double* __restrict__ X, int ldx, const double* __restrict__ Y, int ldy, int K,
     EpiParams<double> p, int nt, const double* skip) {
+    // programmatic dependent launch: the next product's blocks may take their places while this
+    // one runs, and this one touches memory only once its predecessor has finished
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (skip && *skip != 0.0) return;
     __shared__ double rows[2 * SM_T][SM_KC + 1];
     __shared__ double part[SM_G - 1][SM_T * SM_T];
@@ -180,9 +184,18 @@ cdmpt_status gemm_simt(int M, int N, int K, const T* X, int ldx, const T* Y, int
             const int mt = (M + SM_T - 1) / SM_T, nt = (N + SM_T - 1) / SM_T;
             p.sym = (ep.sym && M == N && p.trans_block <= 0) ? 1 : 0;
             const int tiles = p.sym ? nt * (nt + 1) / 2 : mt * nt;
-            k_gemm_small_f64<<<tiles, SM_G * SM_T * SM_T, 0, s>>>(X, ldx, Y, ldy, K, p, nt, skip);
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(tiles);
+            cfg.blockDim = dim3(SM_G * SM_T * SM_T);
+            cfg.stream = s;
+            cudaLaunchAttribute a;
+            a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            a.val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = &a;
+            cfg.numAttrs = 1;
+            cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_small_f64, X, ldx, Y, ldy, K, p, nt, skip);
             count_launch();
-            cudaError_t e = cudaGetLastError();
+            if (e == cudaSuccess) e = cudaGetLastError();
             if (e != cudaSuccess) {
                 set_error(std::string("gemm_simt launch: ") + cudaGetErrorString(e));
                 return CDMPT_ERR_CUDA;
