@@ -57,6 +57,14 @@ cdmpt_status check_device_error(cudaStream_t s) {
     return CDMPT_OK;
 }
 
+cdmpt_status read_error_word(cudaStream_t s, int* pinned_word) {
+    int* w = device_error_word();
+    *pinned_word = DEV_OK;
+    if (w) CDMPT_CUDA_TRY(cudaMemcpyAsync(pinned_word, w, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CDMPT_CUDA_TRY(cudaStreamSynchronize(s));
+    return *pinned_word == DEV_OK ? CDMPT_OK : check_device_error(s);
+}
+
 }  // namespace cdmpt
 
 using namespace cdmpt;
@@ -215,7 +223,7 @@ cdmpt_status cdmpt_create(const cdmpt_opts* opts, cdmpt_handle** out) {
         delete h;
         return s;
     }
-    if (cudaMallocHost((void**)&h->cx.pinned, 64 * sizeof(double)) != cudaSuccess ||
+    if (cudaMallocHost((void**)&h->cx.pinned, (kPinnedScalars + 1) * sizeof(double)) != cudaSuccess ||
         cudaMalloc((void**)&h->dscal, 8 * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         set_error("allocation of handle scalars failed");

@@ -489,8 +489,7 @@ cdmpt_status zero_slots(cdmpt_batch* b, int first, int count) {
 cdmpt_status read_all(cdmpt_batch* b) {
     CDMPT_CUDA_TRY(cudaMemcpyAsync(b->pinned, scal_base(b), (size_t)b->B * kSlots * sizeof(double),
                                    cudaMemcpyDeviceToHost, b->cx.stream));
-    CDMPT_CUDA_TRY(cudaStreamSynchronize(b->cx.stream));
-    return check_device_error(b->cx.stream);
+    return read_error_word(b->cx.stream, (int*)(b->pinned + (size_t)b->B * kSlots));
 }
 
 // Per-system arguments of one grouped CG solve: X (s I + t W) = rhs_scale rhs.
@@ -1390,7 +1389,7 @@ cdmpt_status cdmpt_batch_create(const cdmpt_opts* opts, int B, const int* N, int
     b->stage_slots = 512;
     if (cudaMallocHost((void**)&b->stage_host, b->slot_bytes * b->stage_slots) != cudaSuccess ||
         cudaMalloc((void**)&b->stage_dev, b->slot_bytes * b->stage_slots) != cudaSuccess ||
-        cudaMallocHost((void**)&b->pinned, (size_t)B * kSlots * sizeof(double)) != cudaSuccess) {
+        cudaMallocHost((void**)&b->pinned, ((size_t)B * kSlots + 1) * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         cdmpt_batch_destroy(b);
         set_error("batch: staging allocation failed");

@@ -86,6 +86,9 @@ enum DeviceError {
 
 int* device_error_word();   // per-device word, zeroed at first use
 cdmpt_status check_device_error(cudaStream_t s);
+// check_device_error through a pinned word, queued behind the caller's own read-backs: one wait
+// for the stream in place of two (the word's copy to pageable memory took a wait of its own)
+cdmpt_status read_error_word(cudaStream_t s, int* pinned_word);
 
 // GEMM launchers (asynchronous).
 template <typename T>

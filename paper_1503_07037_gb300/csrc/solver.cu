@@ -220,8 +220,7 @@ template <typename T>
 cdmpt_status Solver<T>::read_scalars(Context& cx, const double* dev, int count) {
     CDMPT_CUDA_TRY(cudaMemcpyAsync(cx.pinned, dev, count * sizeof(double), cudaMemcpyDeviceToHost,
                                    cx.stream));
-    CDMPT_CUDA_TRY(cudaStreamSynchronize(cx.stream));
-    return check_device_error(cx.stream);
+    return read_error_word(cx.stream, (int*)(cx.pinned + kPinnedScalars));
 }
 
 // The mu step of the occupation loop when Newton's step (Eq. NewtRaphs: slope beta Tr[P (I -

@@ -12,6 +12,8 @@
 
 namespace cdmpt {
 
+constexpr int kPinnedScalars = 64;
+
 struct Context {
     cudaStream_t stream = nullptr;
     int engine = CDMPT_GEMM_AUTO;   // float storage only
@@ -24,7 +26,7 @@ struct Context {
     std::vector<int> ev_engine;     // engine of pair i
     std::vector<double> ev_flops;   // algorithmic flops of pair i
     size_t ev_used = 0;
-    double* pinned = nullptr;       // host scalar readback (64 doubles)
+    double* pinned = nullptr;       // host scalar readback (kPinnedScalars doubles and a word)
     // phase boundaries of a solve (profile mode): start, after the occupation sweeps,
     // after the refinement, after the response, after dP0/dmu, end
     cudaEvent_t ph[6] = {};
