@@ -222,7 +222,16 @@ __global__ void __launch_bounds__(tc_threads(KCH), 1)
               const __grid_constant__ GemmProblem single, const GemmProblem* groups, int G,
               int total_tiles, int* err) {
     using C = Cfg<BN, STAGES, PASSES>;
-    if (!GROUPED && single.skip != nullptr && *single.skip != 0.0) return;
+    // Programmatic dependent launch (single products): the successor's CTAs may take free SMs and
+    // set up their barriers, tensor memory and descriptors while this product runs; each waits
+    // for its predecessor's end before it touches memory (the flag here, the operands below).
+    if constexpr (!GROUPED) {
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        if (single.skip != nullptr) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            if (*single.skip != 0.0) return;
+        }
+    }
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -336,6 +345,7 @@ __global__ void __launch_bounds__(tc_threads(KCH), 1)
             fill[i] = e;
         }
     }
+    if constexpr (!GROUPED) asm volatile("griddepcontrol.wait;" ::: "memory");
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -706,10 +716,21 @@ cdmpt_status launch(int M, int N, int K, const float* X, const float* Xl, int ld
     pr.p.sym = sym ? 1 : 0;
     const int tiles = tile_count(BM, BN, M, N, sym);
     const int grid = tiles < sm_count() ? tiles : sm_count();
-    k_gemm_tc<BN, STAGES, PASSES, KCH, false, SCREEN><<<grid, tc_threads(KCH), C::SMEM, s>>>(
-        mx, my, mxl, myl, pr, nullptr, 1, tiles, device_error_word());
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(tc_threads(KCH));
+    cfg.dynamicSmemBytes = C::SMEM;
+    cfg.stream = s;
+    cudaLaunchAttribute a;
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &a;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_tc<BN, STAGES, PASSES, KCH, false, SCREEN>, mx,
+                                       my, mxl, myl, pr, (const GemmProblem*)nullptr, 1, tiles,
+                                       device_error_word());
     count_launch();
-    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_error(std::string("tcgen05 GEMM launch: ") + cudaGetErrorString(e));
         return CDMPT_ERR_CUDA;
