@@ -9,8 +9,9 @@
  *       X_0 = I/2 - 2^-(n+2) beta (H0 - mu I),
  *       X_k = X_{k-1}^2 [X_{k-1}^2 + (I - X_{k-1})^2]^-1,  k = 1..n,
  *     each step a linear solve T X_k = X_{k-1}^2 with
- *     T = 2 X_{k-1}(X_{k-1} - I) + I, by conjugate gradients warm-started
- *     from the previous iterate (Sec. II, Algorithm 1);
+ *     T = 2 X_{k-1}(X_{k-1} - I) + I (Sec. II, Algorithm 1), by a polynomial in
+ *     T of the degree its spectral interval asks for, or by conjugate
+ *     gradients warm-started from the previous iterate;
  *   - the first-order response X^(1) carried through every step with the
  *     same system matrix T (Algorithm 1, order 1);
  *   - the canonical constraint Tr P0 = N_occ on mu (Newton steps on the
@@ -90,7 +91,8 @@ typedef struct {
     int gemm_engine;    /* cdmpt_gemm_engine. FP64 storage: AUTO or TC_OZAKI (FP64 Ozaki
                            products on the tensor cores) or SIMT (CUDA-core DFMA) */
     double cg_tol;      /* CG stop: ||R||_F <= cg_tol * ||RHS||_F; <= 0 selects the default */
-    int cg_maxit;       /* CG iteration cap per solve */
+    int cg_maxit;       /* cap per solve on CG iterations and on the degree of the polynomials
+                           that replace them; a cap below a solve's degree selects CG */
     int refine_rounds;  /* residual-refinement rounds (MIXED_* only) */
     double occ_tol;     /* stop when |Tr P0 - N_occ| <= occ_tol; <= 0 selects N * 1e-12 (FP64)
                            or N * 1e-7 (otherwise) */
@@ -149,11 +151,11 @@ typedef struct {
 typedef struct {
     int N, D, n;                   /* sizes of the last solve */
     int mu_iterations;             /* occupation sweeps (0th-order recursions) */
-    int cg_iterations_sweeps;      /* CG iterations summed over all sweeps */
+    int cg_iterations_sweeps;      /* CG iterations, or polynomial degrees, summed over all sweeps */
     int cg_iterations_last_sweep;  /* CG iterations of the final sweep */
-    int cg_iterations_response;    /* CG iterations of the response pass */
+    int cg_iterations_response;    /* CG iterations of the response pass (0: closed form) */
     int cg_iterations_q;           /* CG iterations of the dP/dmu solve */
-    int cg_iterations_refine;      /* CG iterations of the refinement */
+    int cg_iterations_refine;      /* CG iterations, or closed-form corrections, of the refinement */
     int gemm_launches;             /* GEMM kernel launches */
     int kernel_launches;           /* all kernel launches of this library */
     double gemm_flops;             /* algorithmic GEMM flops, sum of 2 M N K */
@@ -351,8 +353,8 @@ cdmpt_status cdmpt_response1(cdmpt_handle* h, int D, const double* H1, double* P
  * P2: D x N x N (row-major FP64), may be NULL. mu2, omega3: host arrays of D
  * doubles, may be NULL. gradH0: N x N, may be NULL. P2 and gradH0 are host or device
  * memory per on_device. The call runs, per direction, one joint forward sweep
- * of orders 1 and 2 with the known mu1 (eight products and two CG solves per
- * step) in the precision of the solve.
+ * of orders 1 and 2 with the known mu1 (eleven products per step) in the
+ * precision of the solve.
  * Errors: ERR_ARG (no solve yet, no directions), ERR_CG_MAXITER,
  * ERR_NO_CONVERGENCE, ERR_OOM, ERR_CUDA. */
 cdmpt_status cdmpt_response2(cdmpt_handle* h, const double* w, double* P2, double* mu2,
