@@ -1023,12 +1023,12 @@ cdmpt_status hp_fork_lanes(cdmpt_batch* b, const std::vector<char>& active, int*
     return CDMPT_OK;
 }
 
-// B_k = Z_{k+1} Z_k (sy.S.x) from four Ozaki digits of the pair-stored trajectory for the flagged
+// B_k = Z_{k+1} Z_k (sy.S.x) from Ozaki digits of the pair-stored trajectory for the flagged
 // systems (see Solver::step_product), on side lanes.
 cdmpt_status step_product_hp(cdmpt_batch* b, int k, const std::vector<char>& active) {
     int L = 0;
     CDMPT_TRY(hp_fork_lanes(b, active, &L));
-    constexpr int nd = 4;
+    constexpr int nd = kOzDigits;
     int j = 0;
     for (int i = 0; i < b->B; ++i) {
         if (!active[i]) continue;

@@ -1420,15 +1420,16 @@ bool Solver<T>::closed_tangent(const cdmpt_opts& o) const {
 // every direction of every later step carries on, and the split product has a bias of about
 // -1.5e-7 (tensor-core accumulation truncates): on the mixed precision's 16^3 lattice it alone
 // took the P1 error from 3.1e-7 to 9.2e-7. So the steps that are refined with FP64-class
-// residuals (k >= k_hp) and the two before them (||B|| above about 0.03) form B_k from four
-// Ozaki digits of the pair-stored trajectory (2^-31
-// of the row maxima, ten BF16 products on upper-triangle tiles; the other products of the step
-// keep the split form); the digits of Z_{k+1} serve the next step as those of its Z_k.
+// residuals (k >= k_hp) and the two before them (||B|| above about 0.03) form B_k from the
+// Ozaki digits of the pair-stored trajectory (2^-39 of the row maxima, fifteen BF16 products on
+// upper-triangle tiles; the other products of the step keep the split form); the digits of
+// Z_{k+1} serve the next step as those of its Z_k. Four digits (2^-31, ten products) left a P1
+// error of 4.0e-7 at N = 4096 and 4.5e-7 at N = 5508 (beta 60), five leave 3.6e-7 and 3.8e-7.
 template <typename T>
 cdmpt_status Solver<T>::step_product(Context& cx, int k, int engine) {
     if constexpr (sizeof(T) == 4) {
         if (pairs_ && Z_[k].xl && k_hp_ < last_n_ && k >= k_hp_ - 2) {
-            constexpr int nd = 4;
+            constexpr int nd = kOzDigits;
             for (int j = k; j <= k + 1; ++j) {
                 if (oz_step_[j & 1] == j) continue;
                 CDMPT_TRY(oz_slice(Z_[j].x, Z_[j].xl, N_, N_, ld, oz_[j & 1], cx.stream, nd));
