@@ -63,7 +63,12 @@ typedef enum {
 typedef enum {
     CDMPT_FP64 = 0,       /* FP64 storage, FP64 products (tensor-core Ozaki slicing into seven
                              BF16 digits on sm_103, or CUDA-core DFMA with CDMPT_GEMM_SIMT) */
-    CDMPT_FP32 = 1,       /* FP32 storage, FP32-accurate products (3xTF32 on tcgen05 by default) */
+    CDMPT_FP32 = 1,       /* FP32 storage, FP32-accurate products (3xTF32 on tcgen05 by default).
+                             With perturbations that are large against H0 (sqrt(N) / 5 times the
+                             larger of |Tr H0| / N and an eighth of the spectral interval, as the
+                             dipole of a long chain) the solve refines its trajectory as
+                             MIXED_TF32 does, since mu1 needs more than FP32 there; an engine
+                             asked for by name, checkpoints or too little memory leave it out */
     CDMPT_MIXED_TF32 = 2, /* one-pass TF32 products for the occupation sweeps; iterative
                              refinement of the pair-stored (hi + lo FP32) trajectory with
                              split-TF32 residuals on the early steps and FP64-class

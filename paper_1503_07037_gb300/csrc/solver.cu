@@ -65,6 +65,7 @@ enum Slot {
     S_TRZ1 = 16,    // Tr Z1_d (d < 16)
     S_ALPHA = 32,   // sum P1_d * H1_d (d < 16)
     S_FE = 48,      // free energy and Omega terms: traces and dots (5 slots)
+    S_QH = 48,      // sum Q * H1_d (d < 16), in a solve
     S_NSLOTS = 64
 };
 constexpr int kMaxD = 16;
@@ -72,6 +73,7 @@ constexpr int kMaxD = 16;
 
 template <typename T>
 Solver<T>::~Solver() {
+    cudaFree(h1_sums_);
     for (void* p : allocs_) cudaFree(p);
 }
 
@@ -661,11 +663,17 @@ cdmpt_status Solver<T>::init_z0(Context& cx, const double* H0, double mu, double
 // First-order start of the Fermi-Dirac-exact variant: Z1_0 = Dtanh(Y)[Y1] for the stacked
 // directions Y1_d = -s2 H1_d (mu1 = 0; the mu1 term is added through Q afterwards).
 template <typename T>
-cdmpt_status Solver<T>::init_z1(Context& cx, const double* H1, int D, T* out, T* out_hi,
-                                T* out_lo) {
-    CDMPT_TRY(Ew<T>::init_z(Z1b_.x, H1, N_, ld, ld, D, -last_s2_, 0.0, cx.stream, Z1b_.hi,
-                            Z1b_.lo));
-    return tanh_tangent(cx, D, out, out_hi, out_lo);
+cdmpt_status Solver<T>::init_z1(Context& cx, const double* H1, int D, const double* shift,
+                                T* out, T* out_hi, T* out_lo) {
+    T* x = fdx_ ? Z1b_.x : out;
+    T* hi = fdx_ ? Z1b_.hi : out_hi;
+    T* lo = fdx_ ? Z1b_.lo : out_lo;
+    for (int d = 0; d < D; ++d) {
+        const size_t o = (size_t)d * blk_;
+        CDMPT_TRY(Ew<T>::init_z(x + o, H1 + o, N_, ld, ld, 1, -last_s2_, shift[d], cx.stream,
+                                hi ? hi + o : nullptr, lo ? lo + o : nullptr));
+    }
+    return fdx_ ? tanh_tangent(cx, D, out, out_hi, out_lo) : CDMPT_OK;
 }
 
 // out_d = Dtanh(Y)[E_d] for the stacked symmetric directions E_d held in Z1b_ (with its TF32
@@ -982,7 +990,7 @@ cdmpt_status Solver<T>::step0(Context& cx, int k, int engine, double tol, int ma
     // row) and screened products; a caller's cap on iterations caps the degree as well.
     const double zb = zbound_[k];
     InversePoly p;
-    if (!(screen_tau_ > 0.f) && engine != CDMPT_GEMM_TC_BF16 &&
+    if (closed_ok_ && !(screen_tau_ > 0.f) && engine != CDMPT_GEMM_TC_BF16 &&
         p.fit(1.0, 0.0, zb * zb, 0.5 * tol, std::min(maxit, sizeof(T) == 8 ? 20 : 16))) {
         Epilogue<T> ep;
         ep.beta = 2.0;
@@ -1351,7 +1359,7 @@ cdmpt_status Solver<T>::compute_q(Context& cx) {
     double rhs_scale = 1.0;
     bool hp_rhs = false;
     if constexpr (sizeof(T) == 4) {
-        if (pairs_ && Z_[n].xl) {
+        if (refined_ && Z_[n].xl) {
             CDMPT_TRY(oz_slice(Z_[n].x, Z_[n].xl, N_, N_, ld, oz_[0], cx.stream));
             OzEpi ep;
             ep.sym = 1;   // I - Z_n Z_n: upper-triangle tiles, mirrored
@@ -1428,7 +1436,7 @@ bool Solver<T>::closed_tangent(const cdmpt_opts& o) const {
 template <typename T>
 cdmpt_status Solver<T>::step_product(Context& cx, int k, int engine) {
     if constexpr (sizeof(T) == 4) {
-        if (pairs_ && Z_[k].xl && k_hp_ < last_n_ && k >= k_hp_ - 2) {
+        if (refined_ && Z_[k].xl && k_hp_ < last_n_ && k >= k_hp_ - 2) {
             constexpr int nd = kOzDigits;
             for (int j = k; j <= k + 1; ++j) {
                 if (oz_step_[j & 1] == j) continue;
@@ -1517,7 +1525,7 @@ cdmpt_status Solver<T>::vjp_p0(Context& cx, const double* G0, double* grad, doub
     Buf<T>& VT = Z1b_;
     Buf<T>& M1T = A1_;
     Buf<T>& B = RHS_;
-    const bool closed = closed_tangent(o);
+    const bool closed = closed_tangent(o) && closed_ok_;
     oz_step_[0] = oz_step_[1] = -1;
     if (closed) {   // the tangent of a step is self-adjoint: Zh_k = tangent_step(Zh_{k+1})
         Buf<T>* cur = &Z1a_;
@@ -1659,7 +1667,8 @@ cdmpt_status Solver<T>::orders(Context& cx, const double* H1d, const double* H2d
     const cdmpt_opts& o = last_opts_;
     auto cur = [&](int q) -> Buf<T>& { return zo_[q - 1][cur_[q - 1]]; };
     auto nxt = [&](int q) -> Buf<T>& { return zo_[q - 1][1 - cur_[q - 1]]; };
-    auto mu_of = [&](int q) { return q < m ? mus[q - 1] : 0.0; };
+    // mus[m - 1]: where the unknown mu^(m) is counted from (0, or the mean of H1's diagonal)
+    auto mu_of = [&](int q) { return mus[q - 1]; };
     for (int q = 1; q <= m; ++q) cur_[q - 1] = 0;
     // the linear starts Y^(q) = -s2 (H^(q) - mu^(q) I); the Fermi-Dirac-exact start keeps them
     // in the next-iterate buffers and maps them through the Taylor coefficients of tanh
@@ -1682,7 +1691,7 @@ cdmpt_status Solver<T>::orders(Context& cx, const double* H1d, const double* H2d
     }
     if (fdx_) CDMPT_TRY(tanh_taylor(cx, m));
     int hint[3] = {1, 1, 1};
-    const bool closed = closed_tangent(o);
+    const bool closed = closed_tangent(o) && closed_ok_;
     oz_step_[0] = oz_step_[1] = -1;
     if (closed && m == 1) {   // first order alone: the tangent of each step
         for (int k = 0; k < n; ++k) {
@@ -1823,14 +1832,21 @@ cdmpt_status Solver<T>::higher(Context& cx, const double* H1, int D, int m, cons
         const double* H1d = H1 + (size_t)d * blk_;
         const double* H2d = H2 ? H2 + (size_t)d * blk_ : nullptr;
         const double* H3d = H3 ? H3 + (size_t)d * blk_ : nullptr;
-        double mus[2] = {m > 1 ? (mu1s ? mu1s[d] : last_mu1_[d]) : 0.0, 0.0};
+        double mus[3] = {m > 1 ? (mu1s ? mu1s[d] : last_mu1_[d]) : 0.0, 0.0, 0.0};
+        if (m == 1 && sizeof(T) == 4 && !gc && closed_tangent(o) && closed_ok_) {
+            CDMPT_CUDA_TRY(cudaMemsetAsync(sc_ + S_TRQ + 1, 0, sizeof(double), cx.stream));
+            CDMPT_TRY(Ew<double>::trace(H1d, N, ld, 1, sc_ + S_TRQ + 1, cx.stream));
+            CDMPT_TRY(read_scalars(cx, sc_, S_NSLOTS));
+            mus[0] = cx.pinned[S_TRQ + 1] / N;
+        }
         for (int q = std::min(m, 2); q <= m; ++q) {
             CDMPT_TRY(orders(cx, H1d, H2d, H3d, q, mus));
             Buf<T>& Zq = zo_[q - 1][cur_[q - 1]];
             CDMPT_CUDA_TRY(cudaMemsetAsync(sc_ + S_TRQ + 1, 0, sizeof(double), cx.stream));
             CDMPT_TRY(Ew<T>::trace(Zq.x, N, ld, 1, sc_ + S_TRQ + 1, cx.stream));
             CDMPT_TRY(read_scalars(cx, sc_, S_NSLOTS));
-            if (sizeof(T) == 4 && closed_tangent(o) && !std::isfinite(cx.pinned[S_TRQ + 1])) {
+            if (sizeof(T) == 4 && closed_tangent(o) && closed_ok_ &&
+                !std::isfinite(cx.pinned[S_TRQ + 1])) {
                 set_error("the response met a non-finite value: no solution of its linear systems");
                 return CDMPT_ERR_CG_MAXITER;
             }
@@ -1839,7 +1855,13 @@ cdmpt_status Solver<T>::higher(Context& cx, const double* H1, int D, int m, cons
                 mus[q - 1] = muq;
                 continue;
             }
-            if (mu_out) mu_out[d] = muq;
+            if (mu_out) mu_out[d] = muq + mus[m - 1];
+            if (mu_out && m == 1 && q_exact()) {   // as in solve()
+                CDMPT_CUDA_TRY(cudaMemsetAsync(sc_ + S_QH, 0, sizeof(double), cx.stream));
+                CDMPT_TRY(Ew<T>::dot_h(Qmu_.x, H1d, N, ld, ld, sc_ + S_QH, cx.stream));
+                CDMPT_TRY(read_scalars(cx, sc_, S_NSLOTS));
+                mu_out[d] = cx.pinned[S_QH] / trQ;
+            }
             // Z^(m) += 2 mu^(m) Q  (P^(m) = Z^(m) / 2)
             if (!gc) CDMPT_TRY(Ew<T>::axpby(Zq.x, Qmu_.x, blk_, 2.0 * muq, 1.0, nullptr, cx.stream));
             if (omega) {
@@ -2129,6 +2151,18 @@ cdmpt_status Solver<T>::free_energy(Context& cx, double* omega, double* grad) {
     return check_device_error(cx.stream);
 }
 
+// FP32 precision and perturbations that are large against H0. mu1 is the average of H1's level
+// elements h_i over the few levels near mu, so errors of about 2e-6 of each level's weight (the
+// products' truncation, the rounding of Z_k) leave an error of 2e-6 h_rms / sqrt(levels) in it,
+// whatever mu1 and mu are themselves: against mu it is 1e-6 and more for the dipole of a long chain
+// or a wide band, 1e-8 to 2e-7 for the dipole of a three-dimensional cell (chains and banded
+// matrices of N = 60 - 1700, beta 5 - 80: 21 of 70 above 1e-6; refined 0 .. 2). Solves with a
+// perturbation of h_rms > sqrt(N) / 5 energy units (the mean level, or an eighth of the spectral
+// interval) therefore refine the trajectory as MIXED_TF32 does. Both groups are far from the
+// line: chains of 64 to 1700 sites 1.1 to 6, lattices of 4^3 to 16^3 0.03 to 0.08.
+// Where the refinement is not to be had (checkpoints, an engine asked for by name, no memory, no
+// convergence), such solves run by CG: its sweeps and response share their products' errors, and
+// these cancel in mu1 better than those of the closed forms do.
 template <typename T>
 cdmpt_status Solver<T>::solve(Context& cx, const double* H0, const double* H1, int N, int D,
                               double gmin, double gmax, double trH0, const cdmpt_opts& o,
@@ -2139,8 +2173,68 @@ cdmpt_status Solver<T>::solve(Context& cx, const double* H0, const double* H1, i
         set_error("at most 16 perturbation directions per solve");
         return CDMPT_ERR_ARG;
     }
+    auto run = [&](const cdmpt_opts& opts, Form form) {
+        return solve_as(cx, H0, H1, N, D, gmin, gmax, trH0, opts, beta, nocc, n, P0, P1, mu_out,
+                        mu1_out, out_on_device, alpha_out, form);
+    };
+    h1_mean_.assign(std::max(D, 0), 0.0);
+    if (sizeof(T) == 8) return run(o, Form::kPlain);
+    const bool fp32 = o.precision == CDMPT_FP32;
+    bool wide = false;
+    if (D > 0 && !o.grand_canonical) {
+        if (!h1_sums_ &&
+            cudaMalloc((void**)&h1_sums_, 2 * kMaxD * sizeof(double)) != cudaSuccess) {
+            cudaGetLastError();
+            set_error("device allocation of the perturbations' sums failed");
+            return CDMPT_ERR_OOM;
+        }
+        const int ldh = (N + 31) / 32 * 32;
+        const size_t blk = (size_t)N * ldh;
+        CDMPT_CUDA_TRY(cudaMemsetAsync(h1_sums_, 0, 2 * kMaxD * sizeof(double), cx.stream));
+        CDMPT_TRY(Ew<double>::trace(H1, N, ldh, D, h1_sums_, cx.stream));
+        for (int d = 0; d < D; ++d)
+            CDMPT_TRY(Ew<double>::dot(H1 + d * blk, H1 + d * blk, blk, h1_sums_ + kMaxD + d,
+                                      nullptr, cx.stream));
+        CDMPT_TRY(read_scalars(cx, h1_sums_, 2 * kMaxD));
+        const double unit = std::max(std::fabs(trH0) / N, (gmax - gmin) / 8.0);
+        for (int d = 0; d < D; ++d) {
+            const double mean = cx.pinned[d] / N;
+            h1_mean_[d] = mean;
+            // h_rms^2 / N, with h_rms^2 = ||H1 - mean I||_F^2 / N
+            const double r = std::max(cx.pinned[kMaxD + d] / N - mean * mean, 0.0) / N;
+            wide = wide || std::sqrt(r) > 0.2 * unit;
+        }
+    }
+    if (!fp32 || !wide) return run(o, Form::kPlain);
+    if (cx.engine == CDMPT_GEMM_AUTO && o.ckpt_stride == 0 && N <= 32768 &&
+        krylov_degree(o.cg_tol) <= o.cg_maxit && tc_supported() &&
+        !(no_memory_N_ > 0 && N >= no_memory_N_)) {
+        cdmpt_opts r = o;
+        r.refine_rounds = 2;
+        r.fp64_residual = 0;
+        const cdmpt_stats before = *cx.st;
+        const cdmpt_status s = run(r, Form::kRefined);
+        if (s != CDMPT_ERR_NO_CONVERGENCE && s != CDMPT_ERR_CG_MAXITER && s != CDMPT_ERR_OOM)
+            return s;
+        if (s == CDMPT_ERR_OOM) no_memory_N_ = N;
+        *cx.st = before;
+        cx.ev_used = 0;
+        for (bool& b : cx.ph_set) b = false;
+    }
+    return run(o, Form::kCg);
+}
+
+template <typename T>
+cdmpt_status Solver<T>::solve_as(Context& cx, const double* H0, const double* H1, int N, int D,
+                                 double gmin, double gmax, double trH0, const cdmpt_opts& o,
+                                 double beta, double nocc, int n, double* P0, double* P1,
+                                 double* mu_out, double* mu1_out, int out_on_device,
+                                 double* alpha_out, Form form) {
     const bool bf16 = sizeof(T) == 4 && o.precision == CDMPT_MIXED_BF16;
-    const bool mixed = sizeof(T) == 4 && (o.precision == CDMPT_MIXED_TF32 || bf16);
+    const bool mixed = sizeof(T) == 4 && (o.precision == CDMPT_MIXED_TF32 || bf16 ||
+                                          form == Form::kRefined);
+    refined_ = mixed;
+    closed_ok_ = form != Form::kCg;
     if (mixed && cx.engine == CDMPT_GEMM_SIMT) {
         set_error("mixed precision needs the tcgen05 engines");
         return CDMPT_ERR_ARG;
@@ -2207,6 +2301,7 @@ cdmpt_status Solver<T>::solve(Context& cx, const double* H0, const double* H1, i
     bool converged = false;
     double trP = 0, zz = 0;
     double e_lo = 0.0, e_hi = 0.0;   // occupation errors at lo and hi once a sweep set them
+    bool closer = false;
     for (int it = 0; it < o.mu_maxit; ++it) {
         int iters = 0;
         CDMPT_TRY(sweep(cx, H0, mu, s2, o, n, fast, sweep_tol, &iters));
@@ -2219,8 +2314,16 @@ cdmpt_status Solver<T>::solve(Context& cx, const double* H0, const double* H1, i
         st.trace_P0 = trP;
         st.occupation_error = std::fabs(err);
         if (std::fabs(err) <= occ_tol_sweep) {
-            converged = true;
-            break;
+            // A trajectory that is not refined: the trace of one form of the sweep differs from
+            // another's by about 1e-8 N, so an error close under the tolerance N 1e-7 takes one
+            // more sweep, as it would in the form whose trace lies beyond it (P1 of a 9 x 5 x 5
+            // lattice at beta 15 stopped at 0.93 of the tolerance: 2.4e-6, one sweep later 6e-7)
+            if (sizeof(T) == 8 || mixed || gc || closer || !closed_ok_ || o.occ_tol > 0 ||
+                it + 1 == o.mu_maxit || std::fabs(err) <= 0.7 * occ_tol) {
+                converged = true;
+                break;
+            }
+            closer = true;
         }
         if (err > 0) {
             hi = mu;
@@ -2233,7 +2336,10 @@ cdmpt_status Solver<T>::solve(Context& cx, const double* H0, const double* H1, i
         double mu_new = slope > 0 ? mu - err / slope : lo - 1.0;
         if (!(mu_new > lo && mu_new < hi))
             mu_new = next_mu_outside_newton(lo, hi, e_lo, e_hi);
-        if (mu_new == mu) break;
+        if (mu_new == mu) {
+            converged = closer && std::fabs(err) <= occ_tol;
+            break;
+        }
         mu = mu_new;
     }
     if (!converged) {
@@ -2265,7 +2371,8 @@ cdmpt_status Solver<T>::solve(Context& cx, const double* H0, const double* H1, i
         // follow) every pass forms the residuals of steps k >= k_hp with Ozaki-sliced
         // products, so that no occupation is measured on a trajectory carrying the split
         // products' bias
-        bool done = false, hp_phase = false;
+        bool done = false, hp_phase = false, tightened = false;
+        int newton = 0;
         int hp_passes = 0;
         for (int pass = 0; pass < min_pass + (bf16 ? 10 : 6) + 4 && !done; ++pass) {
             int iters = 0;
@@ -2284,12 +2391,22 @@ cdmpt_status Solver<T>::solve(Context& cx, const double* H0, const double* H1, i
                               : std::max(1e-9 * N, pass + 1 >= min_pass ? 1e-7 * std::sqrt((double)N)
                                                                          : 0.0);
             const bool occ_ok = std::fabs(err) <= tol_ref;
+            // What an occupation error does to the response goes with beta |dmu| = |err| / S,
+            // S = sum p (1 - p): with few levels near mu (S below 20) tol_ref alone leaves up to
+            // 1e-6. One more pass where it is above 2e-7 and above the traces' noise
+            bool tight = true;
             if (hp_phase) {
+                const double S = 0.25 * (N - zz);
+                tight = gc || o.occ_tol > 0 || tightened ||
+                        std::fabs(err) <= std::max(2e-7 * S, 1e-10 * N);
                 if (occ_ok && pass + 1 >= min_pass) {
-                    done = true;
-                    break;
+                    if (tight || !(S > 0.05)) {
+                        done = true;
+                        break;
+                    }
+                    tightened = true;
                 }
-                if (++hp_passes >= 4) break;
+                if (++hp_passes >= 4 + (tightened ? 1 : 0)) break;
             } else {
                 // the pass started from relative step residuals below 1e-6, so it left them
                 // at about 1e-9 or at the split-TF32 floor (or, after three extra passes,
@@ -2314,7 +2431,9 @@ cdmpt_status Solver<T>::solve(Context& cx, const double* H0, const double* H1, i
                     }
                 }
             }
-            if (!occ_ok) {   // Newton step on mu; Z_0 = -s2 (H - mu I) moves by s2 dmu I
+            if (!occ_ok || !tight) {   // Newton step on mu; Z_0 = -s2 (H - mu I) moves by s2 dmu I
+                // an FP32 solve counts it against its cap on sweeps
+                if (form == Form::kRefined && st.mu_iterations + ++newton > o.mu_maxit) break;
                 const double slope = 0.25 * beta * (N - zz);
                 const double dmu = slope > 0 ? -err / slope : 0.0;
                 mu += dmu;
@@ -2349,13 +2468,13 @@ cdmpt_status Solver<T>::solve(Context& cx, const double* H0, const double* H1, i
         const size_t count = (size_t)rows * ld;
         Buf<T>* Z1 = &Z1a_;
         Buf<T>* Z1n = &Z1b_;
-        if (fdx_)
-            CDMPT_TRY(init_z1(cx, H1, D, Z1->x, Z1->hi, Z1->lo));
-        else
-            CDMPT_TRY(Ew<T>::init_z(Z1->x, H1, N, ld, ld, D, -s2, 0.0, cx.stream, Z1->hi,
-                                    Z1->lo));
+        const bool closed = closed_tangent(o) && closed_ok_;
+        // FP32 storage, canonical: the response to H1 - c I, c the mean of its diagonal, with mu1
+        // counted from c: Tr P1|0 then carries no part that the mu1 term takes away again
+        double shift[kMaxD] = {};
+        for (int d = 0; d < D && sizeof(T) == 4 && closed && !gc; ++d) shift[d] = h1_mean_[d];
+        CDMPT_TRY(init_z1(cx, H1, D, shift, Z1->x, Z1->hi, Z1->lo));
         int total = 0, hint = 1;
-        const bool closed = closed_tangent(o);
         oz_step_[0] = oz_step_[1] = -1;
         for (int k = 0; k < n && closed; ++k) {
             CDMPT_TRY(need(cx, k));
@@ -2442,19 +2561,27 @@ cdmpt_status Solver<T>::solve(Context& cx, const double* H0, const double* H1, i
                                        cx.stream));
         if (!gc) CDMPT_TRY(Ew<T>::trace(Qmu_.x, N, ld, 1, sc_ + S_TRQ, cx.stream));
         CDMPT_TRY(Ew<T>::trace(Z1->x, N, ld, D, sc_ + S_TRZ1, cx.stream));
+        const bool mu1_of_q = q_exact();
+        for (int d = 0; d < D && mu1_of_q; ++d)
+            CDMPT_TRY(Ew<T>::dot_h(Qmu_.x, H1 + (size_t)d * blk_, N, ld, ld, sc_ + S_QH + d,
+                                   cx.stream));
         CDMPT_TRY(read_scalars(cx, sc_, S_NSLOTS));
         const double trQ = cx.pinned[S_TRQ];
         st.trace_Q = trQ;
+        double qh[kMaxD];   // the slots are read back again below
+        for (int d = 0; d < kMaxD; ++d) qh[d] = cx.pinned[S_QH + d];
         for (int d = 0; d < D; ++d) {
             const double trP1 = 0.5 * cx.pinned[S_TRZ1 + d];
             if (closed && sizeof(T) == 4 && !std::isfinite(trP1)) {
                 set_error("the response met a non-finite value: no solution of its linear systems");
                 return CDMPT_ERR_CG_MAXITER;
             }
-            // grand canonical: mu stays fixed, so mu1 = 0 and P1 = Z1 / 2
+            // grand canonical: mu stays fixed, so mu1 = 0 and P1 = Z1 / 2. P1 takes the mu1 (from
+            // the mean) that makes it traceless; the one handed out is Tr[Q H1] / Tr Q where
+            // Q is the more accurate of the two (see q_exact)
             const double mu1 = (!gc && trQ > 0) ? -trP1 / trQ : 0.0;
-            if (mu1_out) mu1_out[d] = mu1;
-            last_mu1_[d] = mu1;
+            last_mu1_[d] = mu1_of_q && trQ > 0 ? qh[d] / trQ : mu1 + shift[d];
+            if (mu1_out) mu1_out[d] = last_mu1_[d];
             // P1 = Z1/2 + mu1 Q  <=>  Z1 += 2 mu1 Q
             if (!gc)
                 CDMPT_TRY(Ew<T>::axpby(Z1->x + (size_t)d * blk_, Qmu_.x, blk_, 2.0 * mu1, 1.0,

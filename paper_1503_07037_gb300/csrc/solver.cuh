@@ -147,6 +147,13 @@ public:
     int ld = 0;
 
 private:
+    // How a solve runs: as its options say; an FP32 solve with the refinement of the mixed
+    // precision; or by CG throughout (see solve() in solver.cu).
+    enum class Form { kPlain, kRefined, kCg };
+    cdmpt_status solve_as(Context& cx, const double* H0, const double* H1, int N, int D,
+                          double gmin, double gmax, double trH0, const cdmpt_opts& o, double beta,
+                          double nocc, int n, double* P0, double* P1, double* mu_out,
+                          double* mu1_out, int out_on_device, double* alpha_out, Form form);
     struct CgArgs {
         // system operator X -> s X + t X W (W symmetric): the step matrix
         // A_k = I + Z_k^2 is applied as X + X W_k so that the small part
@@ -189,7 +196,9 @@ private:
     // directions of H1 (into out, with its TF32 split).
     cdmpt_status init_z0(Context& cx, const double* H0, double mu, double s2, double rho,
                          int engine);
-    cdmpt_status init_z1(Context& cx, const double* H1, int D, T* out, T* out_hi, T* out_lo);
+    // shift: D values, the start belongs to H1_d - shift_d I
+    cdmpt_status init_z1(Context& cx, const double* H1, int D, const double* shift, T* out,
+                         T* out_hi, T* out_lo);
     // out_d = Dtanh(Y)[E_d] for D stacked directions E_d held in Z1b_ (Fermi-Dirac-exact
     // start; the map is self-adjoint, so it also serves the reverse sweep).
     cdmpt_status tanh_tangent(Context& cx, int D, T* out, T* out_hi, T* out_lo);
@@ -201,7 +210,7 @@ private:
     // segment of step k from its checkpoint unless the segment buffers hold it).
     cdmpt_status need(Context& cx, int k);
     // Joint forward sweep of the orders 1..m (m <= 3) for one direction H1d, with
-    // mu^(1..m-1) = mus[0..m-2] known and mu^(m) = 0. Leaves Z^(o)_n in
+    // mu^(1..m) = mus[0..m-1] (mu^(m): where the unknown one is counted from). Leaves Z^(o)_n in
     // zo_[o-1][cur_[o-1]].
     cdmpt_status orders(Context& cx, const double* H1d, const double* H2d, const double* H3d,
                         int m, const double* mus);
@@ -294,6 +303,18 @@ private:
     int cur_[3] = {0, 0, 0};
     bool orders_ready_ = false;
     std::vector<double> last_mu1_;
+    std::vector<double> h1_mean_;    // mean diagonal of the last solve's H1_d (FP32 storage)
+    double* h1_sums_ = nullptr;      // traces and squares of H1_d (device, 32 doubles)
+    int no_memory_N_ = 0;            // smallest N whose pair storage did not fit
+    bool refined_ = false;           // the trajectory is refined (pairs, FP64-class residuals)
+    bool closed_ok_ = true;          // closed forms in place of CG in sweeps and derivatives
+    // Q = dP0/dmu comes from FP64-class products of a refined Z_n: mu1 = Tr[Q H1] / Tr Q is then
+    // good to the rounding of Q, while the split products of the tangent steps leave errors of
+    // 1e-7 of each level's weight in -Tr P1|0 / Tr Q (N = 60 - 1700, chains and banded matrices:
+    // 4e-8 against 1e-8 of the larger of mu and mu1, geometric mean)
+    bool q_exact() const {
+        return refined_ && !last_opts_.grand_canonical && last_opts_.fp64_residual >= 0;
+    }
     // state of the last solve, for the response's Q and the adjoint
     bool traj_valid_ = false, q_valid_ = false;
     double last_beta_ = 0, last_s2_ = 0;
