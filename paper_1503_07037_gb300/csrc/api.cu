@@ -79,6 +79,7 @@ struct cdmpt_handle {
     double* H3 = nullptr;
     double* dscal = nullptr;  // device scalars for set_H (bounds, trace)
     double gmin = 0, gmax = 0, trH0 = 0;
+    bool finite = true;       // no NaN or infinity in H0 and H1
     Solver<float>* sf = nullptr;
     Solver<double>* sd = nullptr;
     Context cx;
@@ -366,12 +367,18 @@ cdmpt_status cdmpt_set_H(cdmpt_handle* h, int N, const double* H0, int D, const 
     if (st != CDMPT_OK) return fail(h, st);
     st = Ew<double>::trace(h->H0, N, ld, 1, h->dscal + 2, s);
     if (st != CDMPT_OK) return fail(h, st);
-    double host[3];
-    CDMPT_CUDA_TRY(cudaMemcpyAsync(host, h->dscal, 3 * sizeof(double), cudaMemcpyDeviceToHost, s));
+    // sums of squares: finite only if every element is
+    st = Ew<double>::dot(h->H0, h->H0, blk, h->dscal + 3, nullptr, s);
+    if (st == CDMPT_OK && D > 0)
+        st = Ew<double>::dot(h->H1, h->H1, D * blk, h->dscal + 4, nullptr, s);
+    if (st != CDMPT_OK) return fail(h, st);
+    double host[5];
+    CDMPT_CUDA_TRY(cudaMemcpyAsync(host, h->dscal, 5 * sizeof(double), cudaMemcpyDeviceToHost, s));
     CDMPT_CUDA_TRY(cudaStreamSynchronize(s));
     h->gmin = host[0];
     h->gmax = host[1];
     h->trH0 = host[2];
+    h->finite = std::isfinite(host[3]) && std::isfinite(host[4]);
     h->solved = false;
     return CDMPT_OK;
 }
@@ -415,6 +422,13 @@ cdmpt_status cdmpt_solve(cdmpt_handle* h, double beta, double nocc, int n, doubl
     const bool gc = h->opts.grand_canonical != 0;   // nocc unused at fixed mu
     if (!(beta > 0) || (!gc && (!(nocc > 0) || !(nocc < h->N))) || n < 1 || n > 60)
         return fail_msg(h, CDMPT_ERR_ARG, "solve: need beta > 0, 0 < nocc < N, 1 <= n <= 60");
+    // the digit products turn a NaN into some number, and the closed forms have no residual that
+    // would show one: the status CG ends with
+    if (!h->finite) {
+        h->solved = false;
+        return fail_msg(h, CDMPT_ERR_CG_MAXITER,
+                        "solve: H0 or H1 holds a non-finite value: no solution of its linear systems");
+    }
     std::memset(&h->st, 0, sizeof(h->st));
     h->st.N = h->N;
     h->st.D = h->D;

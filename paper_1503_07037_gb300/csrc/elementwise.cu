@@ -6,6 +6,7 @@
 // dimension ld (a multiple of 32 elements); columns N..ld-1 hold zero and
 // every kernel here maps zero padding to zero padding.
 #include <cuda_runtime.h>
+#include <math_constants.h>
 
 #include <algorithm>
 #include <mutex>
@@ -215,7 +216,11 @@ __global__ void k_cg_scalar_init(double* sc, double tol2, double tol2_r0, const 
 }
 
 __global__ void k_refine_ratio(double* v) {
-    if (v[1] > 0.0) v[2] = fmax(v[2], sqrt(v[0] / (4.0 * v[1])));
+    // fmax drops a NaN: a residual that is none counts as the worst there is
+    if (!isfinite(v[0]) || !isfinite(v[1]))
+        v[2] = CUDART_INF;
+    else if (v[1] > 0.0)
+        v[2] = fmax(v[2], sqrt(v[0] / (4.0 * v[1])));
     v[0] = v[1] = 0.0;
 }
 

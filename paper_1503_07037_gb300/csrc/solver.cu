@@ -1341,7 +1341,16 @@ cdmpt_status Solver<T>::occupation(Context& cx, int n, double* trP, double* zz) 
     CDMPT_TRY(read_scalars(cx, sc_, S_NSLOTS));
     *trP = 0.5 * (N_ + cx.pinned[S_TRZ]);
     *zz = cx.pinned[S_ZZ];
+    if (!std::isfinite(*trP) || !std::isfinite(*zz)) return non_finite("the recursion");
     return CDMPT_OK;
+}
+
+// The closed forms meet no tolerance, so a NaN or an infinity shows in their traces only; the
+// status is the one CG ends with.
+template <typename T>
+cdmpt_status Solver<T>::non_finite(const char* what) {
+    set_error(std::string(what) + " met a non-finite value: no solution of its linear systems");
+    return CDMPT_ERR_CG_MAXITER;
 }
 
 // Q = dP0/dmu = beta/4 (I - Z_n^2)(I - Z_0^2)^-1 for the stored trajectory,
@@ -1594,12 +1603,12 @@ cdmpt_status Solver<T>::vjp_p0(Context& cx, const double* G0, double* grad, doub
     CDMPT_CUDA_TRY(cudaMemsetAsync(sc_ + S_TRQ, 0, 2 * sizeof(double), cx.stream));
     if (!gc) CDMPT_TRY(Ew<T>::trace(Qmu_.x, N, ld, 1, sc_ + S_TRQ, cx.stream));
     CDMPT_TRY(Ew<T>::trace(Zh_.x, N, ld, 1, sc_ + S_TRQ + 1, cx.stream));
+    CDMPT_CUDA_TRY(cudaMemsetAsync(sc_ + S_QH, 0, sizeof(double), cx.stream));
+    CDMPT_TRY(Ew<double>::dot_h(G0, G0, N, N, N, sc_ + S_QH, cx.stream));
     CDMPT_TRY(read_scalars(cx, sc_, S_NSLOTS));
     const double trQ = cx.pinned[S_TRQ], trZh = cx.pinned[S_TRQ + 1];
-    if (closed && sizeof(T) == 4 && !std::isfinite(trZh)) {
-        set_error("the adjoint sweep met a non-finite value: no solution of its linear systems");
-        return CDMPT_ERR_CG_MAXITER;
-    }
+    if (!std::isfinite(trZh) || !std::isfinite(cx.pinned[S_QH]))
+        return non_finite("the adjoint sweep");
     const double c = (!gc && trQ > 0) ? last_s2_ * trZh / trQ : 0.0;
     CDMPT_TRY(Ew<T>::lincomb(Zh_.x, Zh_.x, -last_s2_, Qmu_.x, c, blk_, cx.stream));
     // optional + p0_weight P0 = p0_weight (I + Z_n) / 2, added in the padded buffer (the
@@ -1839,17 +1848,18 @@ cdmpt_status Solver<T>::higher(Context& cx, const double* H1, int D, int m, cons
             CDMPT_TRY(read_scalars(cx, sc_, S_NSLOTS));
             mus[0] = cx.pinned[S_TRQ + 1] / N;
         }
+        // a NaN in the perturbation (the digit products would turn it into some number)
+        CDMPT_CUDA_TRY(cudaMemsetAsync(sc_ + S_QH + 1, 0, sizeof(double), cx.stream));
+        for (const double* H : {H1d, H2d, H3d})
+            if (H) CDMPT_TRY(Ew<double>::dot(H, H, blk_, sc_ + S_QH + 1, nullptr, cx.stream));
         for (int q = std::min(m, 2); q <= m; ++q) {
             CDMPT_TRY(orders(cx, H1d, H2d, H3d, q, mus));
             Buf<T>& Zq = zo_[q - 1][cur_[q - 1]];
             CDMPT_CUDA_TRY(cudaMemsetAsync(sc_ + S_TRQ + 1, 0, sizeof(double), cx.stream));
             CDMPT_TRY(Ew<T>::trace(Zq.x, N, ld, 1, sc_ + S_TRQ + 1, cx.stream));
             CDMPT_TRY(read_scalars(cx, sc_, S_NSLOTS));
-            if (sizeof(T) == 4 && closed_tangent(o) && closed_ok_ &&
-                !std::isfinite(cx.pinned[S_TRQ + 1])) {
-                set_error("the response met a non-finite value: no solution of its linear systems");
-                return CDMPT_ERR_CG_MAXITER;
-            }
+            if (!std::isfinite(cx.pinned[S_TRQ + 1]) || !std::isfinite(cx.pinned[S_QH + 1]))
+                return non_finite("the response");
             const double muq = gc ? 0.0 : -0.5 * cx.pinned[S_TRQ + 1] / trQ;
             if (q < m) {
                 mus[q - 1] = muq;
@@ -2572,10 +2582,7 @@ cdmpt_status Solver<T>::solve_as(Context& cx, const double* H0, const double* H1
         for (int d = 0; d < kMaxD; ++d) qh[d] = cx.pinned[S_QH + d];
         for (int d = 0; d < D; ++d) {
             const double trP1 = 0.5 * cx.pinned[S_TRZ1 + d];
-            if (closed && sizeof(T) == 4 && !std::isfinite(trP1)) {
-                set_error("the response met a non-finite value: no solution of its linear systems");
-                return CDMPT_ERR_CG_MAXITER;
-            }
+            if (!std::isfinite(trP1)) return non_finite("the response");
             // grand canonical: mu stays fixed, so mu1 = 0 and P1 = Z1 / 2. P1 takes the mu1 (from
             // the mean) that makes it traceless; the one handed out is Tr[Q H1] / Tr Q where
             // Q is the more accurate of the two (see q_exact)

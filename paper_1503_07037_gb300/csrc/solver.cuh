@@ -259,6 +259,7 @@ private:
     int k_hp_ = 0;                   // first step of the FP64-class residuals of the last solve
     cdmpt_status occupation(Context& cx, int n, double* trP, double* zz);
     cdmpt_status compute_q(Context& cx);
+    static cdmpt_status non_finite(const char* what);
     cdmpt_status read_scalars(Context& cx, const double* dev, int count);
     int engine_of(const Context& cx, int override_engine) const;
 
