@@ -408,6 +408,8 @@ __device__ __forceinline__ float epi_block32(const EpiParams<float>& p, int m0, 
                              (p.beta != 0.f ? (uintptr_t)p.C : 0);
         const int lds = p.ldd | (p.beta != 0.f ? p.ldc : 0);
         vec = vec && (al & 15) == 0 && (lds & 3) == 0;
+        // the four-element form follows the diagonal of gamma I by one wrap per four rows
+        vec = vec && (p.gamma == 0.f || p.diag_block >= 4);
     }
     float local;
     if (vec) {

@@ -69,3 +69,26 @@ def test_epilogue_blocks(cuda, cdmpt_lib, engine, M, N, K, pad, off, mode):
     assert abs(dot.item() - s) <= 1e-5 * s
     if mode == "sym":
         assert np.array_equal(out[:, :N], out[:, :N].T)
+
+
+@pytest.mark.parametrize("engine", ["3xtf32", "tf32"])
+@pytest.mark.parametrize("diag", [1, 2, 3, 4, 5, 31])
+@pytest.mark.parametrize("N", [32, 64, 260])
+def test_small_diagonal_blocks(cuda, cdmpt_lib, engine, diag, N):
+    """gamma I on diagonal blocks below, at and above the four rows of one vector step: gamma
+    stands at [m % diag == n], with products and C small against it."""
+    import torch
+    g = np.random.default_rng(N + diag)
+    X = g.standard_normal((N, 32)).astype(np.float32)
+    C = g.standard_normal((N, N)).astype(np.float32)
+    dev = lambda a: torch.from_numpy(a).cuda()
+    D = torch.empty(N * N, dtype=torch.float32, device="cuda")
+    dot = torch.zeros(1, dtype=torch.float64, device="cuda")
+    _call(cdmpt_lib, engine, dev(X), dev(X), D, N, dev(C), 1000.0, diag, 0, dot)
+    X64 = X.astype(np.float64)
+    P, mag = X64 @ X64.T, np.abs(X64) @ np.abs(X64).T
+    eye = 1000.0 * ((np.arange(N)[:, None] % diag) == np.arange(N)[None, :])
+    ref = 0.5 * P - 1.25 * C + eye
+    got = D.cpu().numpy().reshape(N, N).astype(np.float64)
+    tol = EPS[engine] * mag + 2.0 ** -21 * (np.abs(ref) + 1.25 * np.abs(C) + eye + mag / 32)
+    assert np.all(np.abs(got - ref) <= tol), np.argwhere(np.abs(got - ref) > tol)[:4]
