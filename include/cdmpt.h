@@ -62,7 +62,9 @@ typedef enum {
 
 typedef enum {
     CDMPT_FP64 = 0,       /* FP64 storage, FP64 products (tensor-core Ozaki slicing into seven
-                             BF16 digits on sm_103, or CUDA-core DFMA with CDMPT_GEMM_SIMT) */
+                             BF16 digits on sm_103 and, up to N of about 320, 400 for symmetric
+                             results, CUDA-core DFMA; DFMA throughout with CDMPT_GEMM_SIMT,
+                             digits throughout with CDMPT_GEMM_TC_OZAKI) */
     CDMPT_FP32 = 1,       /* FP32 storage, FP32-accurate products (3xTF32 on tcgen05 by default).
                              With perturbations that are large against H0 (sqrt(N) / 5 times the
                              larger of |Tr H0| / N and an eighth of the spectral interval, as the
@@ -88,13 +90,14 @@ typedef enum {
                                  refinement residuals of the mixed precisions (pair-stored
                                  operands, cdmpt_gemm_pair; statistics only there), and every
                                  product of the FP64 precision (seven digits, cdmpt_gemm_f64_tc;
-                                 the default for FP64 on sm_103) */
+                                 AUTO takes it there for all but small products) */
 } cdmpt_gemm_engine;
 
 typedef struct {
     int precision;      /* cdmpt_precision */
-    int gemm_engine;    /* cdmpt_gemm_engine. FP64 storage: AUTO or TC_OZAKI (FP64 Ozaki
-                           products on the tensor cores) or SIMT (CUDA-core DFMA) */
+    int gemm_engine;    /* cdmpt_gemm_engine. FP64 storage: TC_OZAKI (FP64 Ozaki products on the
+                           tensor cores), SIMT (CUDA-core DFMA) or AUTO (DFMA for small products,
+                           else Ozaki) */
     double cg_tol;      /* CG stop: ||R||_F <= cg_tol * ||RHS||_F; <= 0 selects the default */
     int cg_maxit;       /* cap per solve on CG iterations and on the degree of the polynomials
                            that replace them; a cap below a solve's degree selects CG */

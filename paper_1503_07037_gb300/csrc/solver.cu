@@ -359,8 +359,9 @@ cdmpt_status Solver<T>::gemm(Context& cx, int M, int Nc, int K, const Operand<T>
                              int engine_override) {
     int engine = engine_of(cx, engine_override);
     if constexpr (sizeof(T) == 8) {
-        // short FP64 products: DFMA tiles beat slicing plus the digit kernel's latency
-        if (engine == CDMPT_GEMM_TC_OZAKI && small_f64(M, Nc, K, ep.sym && M == Nc))
+        // short FP64 products: DFMA tiles beat slicing plus the digit kernel's latency. A caller
+        // who names the digit engine gets it for every product
+        if (engine == CDMPT_GEMM_TC_OZAKI && cx.engine != CDMPT_GEMM_TC_OZAKI && small_f64(M, Nc, K, ep.sym && M == Nc))
             engine = CDMPT_GEMM_SIMT;
     }
     // flops the product needs: a symmetric result on the tensor-core engines is
