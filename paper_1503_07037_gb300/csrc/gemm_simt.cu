@@ -156,6 +156,10 @@ bool small_f64(int M, int N, int K, bool sym) {
     return (sym ? 0.5 : 1.0) * M * (double)N * K <= 3.4e7;
 }
 
+bool dfma_small_tiles(int M, int N) {
+    return (size_t)((M + BM - 1) / BM) * ((N + BN - 1) / BN) < 304;
+}
+
 template <typename T>
 cdmpt_status gemm_simt(int M, int N, int K, const T* X, int ldx, const T* Y, int ldy, T* D,
                        int ldd, const Epilogue<T>& ep, const double* skip, cudaStream_t s) {
@@ -180,7 +184,7 @@ cdmpt_status gemm_simt(int M, int N, int K, const T* X, int ldx, const T* Y, int
     p.sym = 0;   // every element is computed here
     if constexpr (sizeof(T) == 8) {
         // small matrices: 8 x 8 tiles until the 64 x 64 tiles fill the SMs
-        if ((size_t)((M + BM - 1) / BM) * ((N + BN - 1) / BN) < 304) {
+        if (dfma_small_tiles(M, N)) {
             const int mt = (M + SM_T - 1) / SM_T, nt = (N + SM_T - 1) / SM_T;
             p.sym = (ep.sym && M == N && p.trans_block <= 0) ? 1 : 0;
             const int tiles = p.sym ? nt * (nt + 1) / 2 : mt * nt;

@@ -96,6 +96,9 @@ cdmpt_status gemm_simt(int M, int N, int K, const T* X, int ldx, const T* Y, int
                        int ldd, const Epilogue<T>& ep, const double* skip, cudaStream_t s);
 // Whether an M x N x K FP64 product is short enough for the DFMA tiles of gemm_simt
 bool small_f64(int M, int N, int K, bool sym);
+// Whether gemm_simt<double> takes its 8 x 8 tiles for an M x N result (a symmetric one then on
+// half of them, mirrored)
+bool dfma_small_tiles(int M, int N);
 
 // Block-norm screening of one tcgen05 product X Y^T (M x N, depth K): the bit mask of
 // the k-slices each 128 x 128 output tile computes (see GemmProblem), nmw words per

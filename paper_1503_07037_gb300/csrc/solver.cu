@@ -264,6 +264,24 @@ int Solver<T>::engine_of(const Context& cx, int override_engine) const {
 }
 
 template <typename T>
+typename Solver<T>::Dispatch Solver<T>::dispatch(const Context& cx, int override_engine, int M,
+                                                 int Nc, int K, bool sym) const {
+    Dispatch d{engine_of(cx, override_engine), sym && M == Nc};
+    if constexpr (sizeof(T) == 8) {
+        // short FP64 products: DFMA tiles beat slicing plus the digit kernel's latency. A caller
+        // who names the digit engine gets it for every product that it takes
+        if (d.engine == CDMPT_GEMM_TC_OZAKI &&
+            (M > rows_cap_ || Nc > N_ || K > N_ || K > 16384 ||
+             (cx.engine != CDMPT_GEMM_TC_OZAKI && small_f64(M, Nc, K, d.half))))
+            d.engine = CDMPT_GEMM_SIMT;
+        if (d.engine == CDMPT_GEMM_SIMT) d.half = d.half && dfma_small_tiles(M, Nc);
+    } else {
+        d.half = d.half && d.engine != CDMPT_GEMM_SIMT;
+    }
+    return d;
+}
+
+template <typename T>
 cdmpt_status Solver<T>::oz64_prepare() {
     if (oz64_ready_) return CDMPT_OK;
     const size_t rows[2] = {(size_t)rows_cap_, (size_t)N_};
@@ -357,17 +375,9 @@ template <typename T>
 cdmpt_status Solver<T>::gemm(Context& cx, int M, int Nc, int K, const Operand<T>& X,
                              const Operand<T>& Y, T* D, const Epilogue<T>& ep, const double* skip,
                              int engine_override) {
-    int engine = engine_of(cx, engine_override);
-    if constexpr (sizeof(T) == 8) {
-        // short FP64 products: DFMA tiles beat slicing plus the digit kernel's latency. A caller
-        // who names the digit engine gets it for every product
-        if (engine == CDMPT_GEMM_TC_OZAKI && cx.engine != CDMPT_GEMM_TC_OZAKI && small_f64(M, Nc, K, ep.sym && M == Nc))
-            engine = CDMPT_GEMM_SIMT;
-    }
-    // flops the product needs: a symmetric result on the tensor-core engines is
-    // computed on its upper-triangular tiles only, N (N + 1) K instead of 2 N^2 K
-    const bool sym_tc = ep.sym && M == Nc && (engine != CDMPT_GEMM_SIMT || sizeof(T) == 8);
-    const double flops = sym_tc ? (double)M * (M + 1) * K : 2.0 * M * (double)Nc * K;
+    const Dispatch run = dispatch(cx, engine_override, M, Nc, K, ep.sym);
+    const int engine = run.engine;
+    const double flops = run.half ? (double)M * (M + 1) * K : 2.0 * M * (double)Nc * K;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (cx.profile) {
         while (cx.ev.size() < 2 * (cx.ev_used + 1)) {
@@ -417,8 +427,7 @@ cdmpt_status Solver<T>::gemm(Context& cx, int M, int Nc, int K, const Operand<T>
             s = gemm_tc_f32(engine, M, Nc, K, X, ld, Y, ld, D, ld, ep, skip, cx.stream, psc);
         }
     } else {
-        if (engine == CDMPT_GEMM_TC_OZAKI && M <= rows_cap_ && Nc <= N_ && K <= N_ &&
-            K <= 16384) {
+        if (engine == CDMPT_GEMM_TC_OZAKI) {
             // slice both operands (once when X is Y), then the digit product
             CDMPT_TRY(oz64_prepare());
             CDMPT_TRY(oz64_slice(X.x, M, K, ld, ox64_, skip, cx.stream));
@@ -538,12 +547,13 @@ cdmpt_status Solver<T>::cg(Context& cx, T* X, const CgArgs& a, int* iters_out,
             for (size_t e = ev_first + ran; e < cx.ev_used; ++e) cx.ev_ok[e] = 0;
         }
         if (cx.st) {
-            const bool sym_tc = a.sym && a.rows == N_ && iter_engine != CDMPT_GEMM_SIMT;
+            const Dispatch it_run =
+                dispatch(cx, a.iter_engine, a.rows, N_, N_, a.sym && a.rows == N_);
             const double f =
-                sym_tc ? (double)N_ * (N_ + 1) * N_ : 2.0 * a.rows * (double)N_ * N_;
+                it_run.half ? (double)N_ * (N_ + 1) * N_ : 2.0 * a.rows * (double)N_ * N_;
             cx.st->gemm_launches += ran;
             cx.st->gemm_flops += ran * f;
-            cx.st->tensor_flops += ran * tensor_factor(iter_engine) * f;
+            cx.st->tensor_flops += ran * tensor_factor(it_run.engine) * f;
         }
         if (cx.pinned[CG_DONE] != 0.0) break;
         if (iters >= a.maxit) {
@@ -1008,7 +1018,7 @@ cdmpt_status Solver<T>::step0(Context& cx, int k, int engine, double tol, int ma
             CDMPT_TRY(poly_eval(cx, W_[k], p, 1.0, engine, &E));
         }
         CDMPT_TRY(gemm(cx, N_, N_, N_, Z_[k].op(), E->op(), Z_[k + 1].x, ep, nullptr, engine));
-        if (engine_of(cx, engine) == CDMPT_GEMM_SIMT)   // full tiles, not mirrored
+        if (!dispatch(cx, engine, N_, N_, N_, true).half)   // full tiles, not mirrored
             CDMPT_TRY(Ew<T>::symmetrize(Z_[k + 1].x, N_, ld, 1, cx.stream, Z_[k + 1].hi,
                                         Z_[k + 1].lo));
         *iters += p.degree();
@@ -1994,7 +2004,7 @@ cdmpt_status Solver<T>::logdet(Context& cx, const Buf<T>& M, double a, double b,
         ep.Dlo = Y.lo;
         ep.sym = true;
         CDMPT_TRY(gemm(cx, N, N, N, L.op(), E->op(), Y.x, ep, nullptr, acc));
-        if (engine_of(cx, acc) == CDMPT_GEMM_SIMT)   // full tiles, not mirrored
+        if (!dispatch(cx, acc, N, N, N, true).half)   // full tiles, not mirrored
             CDMPT_TRY(Ew<T>::symmetrize(Y.x, N, ld, 1, cx.stream, Y.hi, Y.lo));
     } else {
         CDMPT_TRY(Ew<T>::axpby(RHS_.x, M.x, blk_, b, 0.0, nullptr, cx.stream));

@@ -262,6 +262,14 @@ private:
     static cdmpt_status non_finite(const char* what);
     cdmpt_status read_scalars(Context& cx, const double* dev, int count);
     int engine_of(const Context& cx, int override_engine) const;
+    // The engine an M x Nc x K product runs on, and whether a symmetric result (sym) is computed
+    // on about half of its tiles and mirrored: N (N + 1) K flops in place of 2 N^2 K.
+    struct Dispatch {
+        int engine;
+        bool half;
+    };
+    Dispatch dispatch(const Context& cx, int override_engine, int M, int Nc, int K,
+                      bool sym) const;
 
     int N_ = 0, D_ = 0, n_ = 0;
     size_t blk_ = 0;                 // N * ld elements

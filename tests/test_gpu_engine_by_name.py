@@ -29,3 +29,16 @@ def test_named_fp64_engine(cuda, cdmpt_lib, N):
     for engine in ("auto", "simt"):
         assert st[engine]["engine_launches"][OZAKI] == 0 and st[engine]["engine_launches"][SIMT] > 0
         assert oracle.rel_frobenius(P[engine], P[OZAKI]) < 1e-10
+
+
+@pytest.mark.parametrize("N,full", [(200, False), (1152, True)])
+def test_dfma_flop_count(cuda, cdmpt_lib, N, full):
+    """DFMA products of symmetric results count N (N + 1) N flops on the 8 x 8 tiles, which compute
+    half of them, and 2 N^3 where the 64 x 64 tiles compute all (18 x 18 tiles and more)."""
+    p = syn.banded_random(N, bandwidth=8, seed=3, beta=4.0, n=8)
+    with cdmpt_lib.Handle(precision="fp64", engine="simt", profile=True) as h:
+        h.set_H(p.H0)
+        h.solve(p.beta, p.nocc, p.n, want_P0=False)
+        st = h.stats()
+    each = st["gemm_flops"] / st["gemm_launches"]
+    assert each == pytest.approx(2.0 * N ** 3 if full else float(N) * (N + 1) * N)
