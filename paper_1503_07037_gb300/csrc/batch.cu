@@ -761,12 +761,17 @@ cdmpt_status poly_step_batch(cdmpt_batch* b, int k, const std::vector<double>& z
                              double tol, int max_degree, int* degree, bool* done) {
     const int G = b->B;
     std::vector<InversePoly> pl(G);
+    // intervals down to 1e-12: below, the powers of a system whose levels coincide underflow in
+    // the coefficients of a shape that another one needs, and an empty interval would send
+    // the whole batch to CG
+    std::vector<double> hi(G);
+    for (int i = 0; i < G; ++i) hi[i] = std::max(zb[i] * zb[i], 1e-12);
     *done = false;
     int s = 0, r = 0, deg = 0;
     for (int i = 0; i < G; ++i) {
         if (b->sys[i].converged) continue;
         InversePoly& q = pl[i];
-        if (!q.fit(1.0, 0.0, zb[i] * zb[i], 0.5 * tol, max_degree)) return CDMPT_OK;
+        if (!q.fit(1.0, 0.0, hi[i], 0.5 * tol, max_degree)) return CDMPT_OK;
         if (q.degree() > deg) {
             deg = q.degree();
             s = q.s;
@@ -776,7 +781,7 @@ cdmpt_status poly_step_batch(cdmpt_batch* b, int k, const std::vector<double>& z
     if (deg == 0 || s > 4) return CDMPT_OK;
     for (int i = 0; i < G; ++i)
         if (!b->sys[i].converged &&
-            !pl[i].fit(1.0, 0.0, zb[i] * zb[i], 0.5 * tol, std::max(max_degree, deg), s, r))
+            !pl[i].fit(1.0, 0.0, hi[i], 0.5 * tol, std::max(max_degree, deg), s, r))
             return CDMPT_OK;
     // one grouped symmetric product; spec(sy, q, g) fills X, Y and the epilogue per system
     auto product = [&](auto spec) -> cdmpt_status {
