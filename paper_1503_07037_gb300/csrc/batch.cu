@@ -1904,6 +1904,25 @@ cdmpt_status cdmpt_batch_solve(cdmpt_batch* b, const double* beta, const double*
             CDMPT_TRY(run_tiles(b, dq, 1, grouped_trace));
             CDMPT_TRY(run_tiles(b, dz, D, grouped_trace));
         }
+        // mu1 = Tr[Q H1] / Tr Q where Q comes from FP64-class products of the refined Z_n (as
+        // Solver::q_exact); P1 takes the shift that makes it traceless
+        const bool mu1_of_q = mixed && b->opts.fp64_residual >= 0;
+        if (mu1_of_q) {
+            CDMPT_TRY(zero_slots(b, B_ALPHA, 16));
+            std::vector<GrpEw> dh;
+            for (int i = 0; i < G; ++i) {
+                Sys& sy = b->sys[i];
+                for (int dd = 0; dd < D; ++dd) {
+                    GrpEw h = ewd(sy.Qmu.x);
+                    h.h = sy.H1 + (size_t)dd * sy.blk;
+                    h.rows = sy.N; h.ld = sy.ld; h.N = sy.N;
+                    h.sc = sy.sc;
+                    h.s0 = B_ALPHA + dd;
+                    dh.push_back(h);
+                }
+            }
+            CDMPT_TRY(run_ew(b, G_DOT_H, dh));
+        }
         CDMPT_TRY(read_all(b));
         {
             std::vector<GrpEw> da, dh;
@@ -1918,7 +1937,11 @@ cdmpt_status cdmpt_batch_solve(cdmpt_batch* b, const double* beta, const double*
                                          "batch: the response met a non-finite value: no solution "
                                          "of its linear systems");
                     const double m1 = trQ > 0 ? -trP1 / trQ : 0.0;
-                    if (mu1) mu1[i * D + dd] = m1;
+                    if (mu1)
+                        mu1[i * D + dd] = mu1_of_q && trQ > 0
+                                              ? b->pinned[i * kSlots + B_ALPHA + dd] /
+                                                    b->pinned[i * kSlots + B_TRQ]
+                                              : m1;
                     GrpEw a = ewd(Z1->x + (size_t)dd * sy.blk, sy.Qmu.x);
                     a.rows = sy.N; a.ld = sy.ld; a.N = sy.N; a.count = (long long)sy.blk;
                     a.s0 = 2.0 * m1 * 0.25 * sy.beta;

@@ -1,4 +1,6 @@
 """Batches at the edges of what the lockstep closed forms are fitted for."""
+import math
+
 import numpy as np
 import pytest
 
@@ -38,3 +40,16 @@ def test_system_whose_levels_coincide(cuda, cdmpt_lib, width, precision):
         ref = oracle.solve(p.H0, p.H1, p.beta, p.nocc, n=n, kind="rec")
         assert oracle.rel_frobenius(r["P0"][i].cpu().numpy(), ref["P0"]) < 1e-5
         assert oracle.rel_frobenius(r["P1"][i].cpu().numpy(), ref["P1"]) < 1e-5
+
+
+def test_mu1_of_wide_perturbations(cuda, cdmpt_lib):
+    """Mixed batch of a wide band and long chains: mu1 to 1e-6 of |(mu, mu1)|, as single solves."""
+    probs = [syn.banded_random(1200, seed=4, beta=27.0, n=14), syn.chain_1d(1477, 3, 13.0, 14),
+             syn.chain_1d(240, 4, 26.0, 14)]
+    for p in probs:
+        p.H0 = p.H0 - 2.0 * np.eye(p.N)
+    r, _ = _solve(cdmpt_lib, probs, "mixed", 14)
+    for i, p in enumerate(probs):
+        ref = oracle.solve(p.H0, p.H1, p.beta, p.nocc, n=14, kind="rec")
+        err = np.abs(r["mu1"][i] - ref["mu1"]).max() / math.hypot(ref["mu"], *ref["mu1"])
+        assert err < 1e-6, (i, err)
