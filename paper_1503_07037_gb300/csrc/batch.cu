@@ -156,6 +156,12 @@ cdmpt_status bfail_msg(cdmpt_batch* b, cdmpt_status s, const std::string& m) {
     return bfail(b, s);
 }
 
+// The status CG ends with where a system holds a NaN or an infinity.
+cdmpt_status non_finite(cdmpt_batch* b, int i) {
+    return bfail_msg(b, CDMPT_ERR_CG_MAXITER, "batch: system " + std::to_string(i) +
+                     " met a non-finite value: no solution of its linear systems");
+}
+
 cdmpt_status grab(cdmpt_batch* b, size_t bytes, void** out) {
     void* p = nullptr;
     if (cudaMalloc(&p, bytes) != cudaSuccess) {
@@ -1513,6 +1519,7 @@ cdmpt_status cdmpt_batch_solve(cdmpt_batch* b, const double* beta, const double*
             if (sy.converged) continue;
             const double trP = 0.5 * (sy.N + b->pinned[i * kSlots + B_TRZ]);
             const double zz = b->pinned[i * kSlots + B_ZZ];
+            if (!std::isfinite(trP) || !std::isfinite(zz)) return non_finite(b, i);
             const double err = trP - sy.nocc;
             double tol = b->opts.occ_tol > 0 ? b->opts.occ_tol : 1e-7 * sy.N;
             // one-pass TF32 traces are good to about 1e-4, and their per-level rounding adds
@@ -1608,6 +1615,7 @@ cdmpt_status cdmpt_batch_solve(cdmpt_batch* b, const double* beta, const double*
                 if (sy.converged) continue;
                 const double trP = 0.5 * (sy.N + b->pinned[i * kSlots + B_TRZ]);
                 const double zz = b->pinned[i * kSlots + B_ZZ];
+                if (!std::isfinite(trP) || !std::isfinite(zz)) return non_finite(b, i);
                 const double err = trP - sy.nocc;
                 // finish mu to 1e-9 N, or to 1e-7 sqrt(N) once the minimum passes are done
                 const double tol = b->opts.occ_tol > 0
@@ -1932,10 +1940,7 @@ cdmpt_status cdmpt_batch_solve(cdmpt_batch* b, const double* beta, const double*
                 const double trQ = 0.25 * sy.beta * b->pinned[i * kSlots + B_TRQ];
                 for (int dd = 0; dd < D; ++dd) {
                     const double trP1 = 0.5 * b->pinned[i * kSlots + B_TRZ1 + dd];
-                    if (closed && !std::isfinite(trP1))
-                        return bfail_msg(b, CDMPT_ERR_CG_MAXITER,
-                                         "batch: the response met a non-finite value: no solution "
-                                         "of its linear systems");
+                    if (!std::isfinite(trP1)) return non_finite(b, i);
                     const double m1 = trQ > 0 ? -trP1 / trQ : 0.0;
                     if (mu1)
                         mu1[i * D + dd] = mu1_of_q && trQ > 0

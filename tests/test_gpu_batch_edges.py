@@ -53,3 +53,15 @@ def test_mu1_of_wide_perturbations(cuda, cdmpt_lib):
         ref = oracle.solve(p.H0, p.H1, p.beta, p.nocc, n=14, kind="rec")
         err = np.abs(r["mu1"][i] - ref["mu1"]).max() / math.hypot(ref["mu"], *ref["mu1"])
         assert err < 1e-6, (i, err)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "mixed"])
+@pytest.mark.parametrize("where", ["H0", "H1"])
+def test_non_finite_system_is_refused(cuda, cdmpt_lib, where, precision):
+    n = 10
+    probs = syn.clusters(B=2, seed=78, sizes=[70, 150], beta=20.0, n=n)
+    A = getattr(probs[1], where)
+    A[..., 2, 5] = A[..., 5, 2] = np.nan
+    with pytest.raises(cdmpt_lib.CdmptError) as e:
+        _solve(cdmpt_lib, probs, precision, n)
+    assert e.value.status == 4
