@@ -82,6 +82,7 @@ struct Sys {
     double beta = 0, nocc = 0, s2 = 0, mu = 0, lo = 0, hi = 0;
     double e_lo = 0, e_hi = 0;   // occupation errors at lo and hi once a sweep set them
     bool converged = false;
+    bool closer = false;     // FP32: one more sweep was asked for (see the occupation loop)
     // mixed refinement: first step of the FP64-class residuals (n: none), whether this
     // system's passes form them yet, and how many such passes it has had
     int khp = 0;
@@ -1476,6 +1477,7 @@ cdmpt_status cdmpt_batch_solve(cdmpt_batch* b, const double* beta, const double*
         sy.mu = std::min(std::max(sy.trH0 / sy.N, sy.lo + 1e-3 * pad), sy.hi - 1e-3 * pad);
         sy.e_lo = sy.e_hi = 0.0;
         sy.converged = false;
+        sy.closer = false;
     }
     // mixed precision: one-pass TF32 sweeps, then split-TF32 refinement (as in cdmpt_solve)
     const bool mixed = b->opts.precision == CDMPT_MIXED_TF32;
@@ -1527,8 +1529,13 @@ cdmpt_status cdmpt_batch_solve(cdmpt_batch* b, const double* beta, const double*
             // finishes mu
             if (mixed) tol = std::max({tol, 1e-5 * sy.N, 5e-4 * std::sqrt((double)sy.N)});
             if (std::fabs(err) <= tol) {
-                sy.converged = true;
-                continue;
+                // close under FP32's tolerance: one more sweep, as in Solver::solve_as
+                if (mixed || sy.closer || b->opts.occ_tol > 0 || std::fabs(err) <= 0.7 * tol ||
+                    sweeps + 1 == b->opts.mu_maxit) {
+                    sy.converged = true;
+                    continue;
+                }
+                sy.closer = true;
             }
             all = false;
             if (err > 0) {
