@@ -30,15 +30,18 @@
 // safeguarded by a bisection bracket. mu1: P1 is linear in mu1 with slope
 // Q = dP0/dmu, which at finite n is exactly beta P0 (I - P0) (I - Z_0^2)^-1;
 // the response runs once with mu1 = 0 and mu1 = -Tr P1|_0 / Tr Q follows in
-// closed form (the fixed point of the mu1 update of Algorithm 1).
+// closed form (the fixed point of the mu1 update of Algorithm 1). The same number is
+// Tr[Q H1] / Tr Q; where Q is formed with FP64-class products that is the one handed out
+// (q_exact), and FP32 storage counts mu1 from the mean diagonal of H1.
 //
 // Mixed precision (CDMPT_MIXED_TF32): the occupation sweeps run with one-pass
 // TF32 products. The converged trajectory is then refined step by step: with
 // Z_k already refined, A_k = I + Z_k^2 and the residual 2 Z_k - Z_{k+1} A_k
-// are formed with split-TF32 (FP32-accurate) products, and the correction of
-// Z_{k+1} is found by CG whose iterations use one-pass TF32 products (mixed-
-// precision iterative refinement of each step's linear system). Between
-// passes a Newton step on mu shifts Z_0 by s2 dmu I. The response then uses
+// are formed with split-TF32 (FP32-accurate) products, from the second pass on with
+// FP64-class ones in the late steps, and the correction of Z_{k+1} takes one-pass TF32
+// products (mixed-precision iterative refinement of each step's linear system). Between
+// passes a Newton step on mu shifts Z_0 by s2 dmu I. FP32 solves of perturbations that are
+// large against H0 are refined the same way (solve). The response then uses
 // split-TF32 products throughout. CDMPT_MIXED_BF16 is the same with the
 // occupation sweeps on BF16-rounded operands (kind::f16, FP32 accumulation).
 #include <cuda_runtime.h>
@@ -1356,6 +1359,36 @@ cdmpt_status Solver<T>::occupation(Context& cx, int n, double* trP, double* zz) 
     return CDMPT_OK;
 }
 
+// mu1_d = Tr[Q H1_d] / Tr Q (see q_exact), carried from the mu of the trajectory to the mu of
+// N_occ: with a perturbation that is large against H0 the occupation error left, |err| / S =
+// beta |dmu| up to 1e-6, would show in mu1 as that times h_rms / sqrt(levels). dQ/dmu =
+// -beta Z_n Q (to the order of 4^-n), one one-pass TF32 product on half of its tiles.
+template <typename T>
+cdmpt_status Solver<T>::mu1_by_q(Context& cx, const double* H1, int D, double* mu1) {
+    const int N = N_;
+    CDMPT_CUDA_TRY(cudaMemsetAsync(sc_ + S_TRQ, 0, (S_NSLOTS - S_TRQ) * sizeof(double), cx.stream));
+    CDMPT_TRY(Ew<T>::axpby(P_.x, Qmu_.x, blk_, 1.0, 0.0, nullptr, cx.stream, P_.hi, P_.lo));
+    Epilogue<T> ep;
+    ep.sym = true;
+    CDMPT_TRY(gemm(cx, N, N, N, Z_[last_n_].op(), P_.op(), RHS_.x, ep, nullptr,
+                   CDMPT_GEMM_TC_TF32));
+    CDMPT_TRY(Ew<T>::trace(Qmu_.x, N, ld, 1, sc_ + S_TRQ, cx.stream));
+    CDMPT_TRY(Ew<T>::trace(RHS_.x, N, ld, 1, sc_ + S_TRQ + 1, cx.stream));
+    for (int d = 0; d < D; ++d) {
+        const double* h = H1 + (size_t)d * blk_;
+        CDMPT_TRY(Ew<T>::dot_h(Qmu_.x, h, N, ld, ld, sc_ + S_QH + d, cx.stream));
+        CDMPT_TRY(Ew<T>::dot_h(RHS_.x, h, N, ld, ld, sc_ + S_ALPHA + d, cx.stream));
+    }
+    CDMPT_TRY(read_scalars(cx, sc_, S_NSLOTS));
+    const double* v = cx.pinned;
+    double dmu = v[S_TRQ] > 0 ? -last_occ_err_ / v[S_TRQ] : 0.0;
+    if (!(last_beta_ * std::fabs(dmu) < 1e-3)) dmu = 0.0;   // mu in a gap: not determined by it
+    const double c = -last_beta_ * dmu;
+    for (int d = 0; d < D; ++d)
+        mu1[d] = (v[S_QH + d] + c * v[S_ALPHA + d]) / (v[S_TRQ] + c * v[S_TRQ + 1]);
+    return CDMPT_OK;
+}
+
 // The closed forms meet no tolerance, so a NaN or an infinity shows in their traces only; the
 // status is the one CG ends with.
 template <typename T>
@@ -1848,6 +1881,8 @@ cdmpt_status Solver<T>::higher(Context& cx, const double* H1, int D, int m, cons
         return CDMPT_ERR_NO_CONVERGENCE;
     }
     if (grad) CDMPT_CUDA_TRY(cudaMemsetAsync(G_.x, 0, blk_ * sizeof(T), cx.stream));
+    double mu1_q[kMaxD] = {};
+    if (m == 1 && q_exact() && D <= kMaxD) CDMPT_TRY(mu1_by_q(cx, H1, D, mu1_q));
     for (int d = 0; d < D; ++d) {
         const double* H1d = H1 + (size_t)d * blk_;
         const double* H2d = H2 ? H2 + (size_t)d * blk_ : nullptr;
@@ -1877,12 +1912,7 @@ cdmpt_status Solver<T>::higher(Context& cx, const double* H1, int D, int m, cons
                 continue;
             }
             if (mu_out) mu_out[d] = muq + mus[m - 1];
-            if (mu_out && m == 1 && q_exact()) {   // as in solve()
-                CDMPT_CUDA_TRY(cudaMemsetAsync(sc_ + S_QH, 0, sizeof(double), cx.stream));
-                CDMPT_TRY(Ew<T>::dot_h(Qmu_.x, H1d, N, ld, ld, sc_ + S_QH, cx.stream));
-                CDMPT_TRY(read_scalars(cx, sc_, S_NSLOTS));
-                mu_out[d] = cx.pinned[S_QH] / trQ;
-            }
+            if (mu_out && m == 1 && q_exact()) mu_out[d] = mu1_q[d];   // as in solve()
             // Z^(m) += 2 mu^(m) Q  (P^(m) = Z^(m) / 2)
             if (!gc) CDMPT_TRY(Ew<T>::axpby(Zq.x, Qmu_.x, blk_, 2.0 * muq, 1.0, nullptr, cx.stream));
             if (omega) {
@@ -2177,7 +2207,7 @@ cdmpt_status Solver<T>::free_energy(Context& cx, double* omega, double* grad) {
 // products' truncation, the rounding of Z_k) leave an error of 2e-6 h_rms / sqrt(levels) in it,
 // whatever mu1 and mu are themselves: against mu it is 1e-6 and more for the dipole of a long chain
 // or a wide band, 1e-8 to 2e-7 for the dipole of a three-dimensional cell (chains and banded
-// matrices of N = 60 - 1700, beta 5 - 80: 21 of 70 above 1e-6; refined 0 .. 2). Solves with a
+// matrices of N = 60 - 1700, beta 5 - 80: 21 of 70 above 1e-6; refined none of 60). Solves with a
 // perturbation of h_rms > sqrt(N) / 5 energy units (the mean level, or an eighth of the spectral
 // interval) therefore refine the trajectory as MIXED_TF32 does. Both groups are far from the
 // line: chains of 64 to 1700 sites 1.1 to 6, lattices of 4^3 to 16^3 0.03 to 0.08.
@@ -2201,7 +2231,7 @@ cdmpt_status Solver<T>::solve(Context& cx, const double* H0, const double* H1, i
     h1_mean_.assign(std::max(D, 0), 0.0);
     if (sizeof(T) == 8) return run(o, Form::kPlain);
     const bool fp32 = o.precision == CDMPT_FP32;
-    bool wide = false;
+    bool wide = wide_ = false;
     if (D > 0 && !o.grand_canonical) {
         if (!h1_sums_ &&
             cudaMalloc((void**)&h1_sums_, 2 * kMaxD * sizeof(double)) != cudaSuccess) {
@@ -2225,6 +2255,7 @@ cdmpt_status Solver<T>::solve(Context& cx, const double* H0, const double* H1, i
             const double r = std::max(cx.pinned[kMaxD + d] / N - mean * mean, 0.0) / N;
             wide = wide || std::sqrt(r) > 0.2 * unit;
         }
+        wide_ = wide;
     }
     if (!fp32 || !wide) return run(o, Form::kPlain);
     if (cx.engine == CDMPT_GEMM_AUTO && o.ckpt_stride == 0 && N <= 32768 &&
@@ -2338,9 +2369,14 @@ cdmpt_status Solver<T>::solve_as(Context& cx, const double* H0, const double* H1
             // A trajectory that is not refined: the trace of one form of the sweep differs from
             // another's by about 1e-8 N, so an error close under the tolerance N 1e-7 takes one
             // more sweep, as it would in the form whose trace lies beyond it (P1 of a 9 x 5 x 5
-            // lattice at beta 15 stopped at 0.93 of the tolerance: 2.4e-6, one sweep later 6e-7)
+            // lattice at beta 15 stopped at 0.93 of the tolerance: 2.4e-6, one sweep later 6e-7).
+            // What the error does to the response goes with beta |dmu| = |err| / S, S = sum
+            // p (1 - p), a quarter of which shows in P1: small systems, where a sweep costs a
+            // millisecond, go on down to 2e-6 S or the trace's own error
+            const double S = 0.25 * (N - zz);
+            const double fine = N <= 512 ? std::max(2e-6 * S, 5e-9 * N) : 0.7 * occ_tol;
             if (sizeof(T) == 8 || mixed || gc || closer || !closed_ok_ || o.occ_tol > 0 ||
-                it + 1 == o.mu_maxit || std::fabs(err) <= 0.7 * occ_tol) {
+                it + 1 == o.mu_maxit || std::fabs(err) <= std::min(fine, 0.7 * occ_tol)) {
                 converged = true;
                 break;
             }
@@ -2394,6 +2430,7 @@ cdmpt_status Solver<T>::solve_as(Context& cx, const double* H0, const double* H1
         // products' bias
         bool done = false, hp_phase = false, tightened = false;
         int newton = 0;
+        double last_step = 0.0;   // of mu, after the last pass
         int hp_passes = 0;
         for (int pass = 0; pass < min_pass + (bf16 ? 10 : 6) + 4 && !done; ++pass) {
             int iters = 0;
@@ -2406,28 +2443,35 @@ cdmpt_status Solver<T>::solve_as(Context& cx, const double* H0, const double* H1
             const double err = gc ? 0.0 : trP - nocc;
             st.trace_P0 = trP;
             st.occupation_error = std::fabs(err);
+            const double step = last_step;
+            last_step = 0.0;
             // finish mu to 1e-9 N, or to 1e-7 sqrt(N) once the minimum passes are done
             const double tol_ref =
                 o.occ_tol > 0 ? occ_tol
                               : std::max(1e-9 * N, pass + 1 >= min_pass ? 1e-7 * std::sqrt((double)N)
                                                                          : 0.0);
             const bool occ_ok = std::fabs(err) <= tol_ref;
-            // What an occupation error does to the response goes with beta |dmu| = |err| / S,
-            // S = sum p (1 - p): with few levels near mu (S below 20) tol_ref alone leaves up to
-            // 1e-6. One more pass where it is above 2e-7 and above the traces' noise
+            // What an occupation error does to P1 goes with beta |dmu| = |err| / S, S = sum
+            // p (1 - p), a quarter of which shows: with few levels near mu (S below 5) tol_ref
+            // alone leaves up to 1e-6. One more pass where it is above 1e-6 and above the traces'
+            // noise (mu1 itself is carried to the mu of N_occ, see mu1_by_q), or where the pass
+            // had a larger Newton step to follow: it leaves some 1e-3 of beta |dmu| in a level's
+            // weight, and few levels average less of it away (chain of 255 sites, beta 49, S = 1:
+            // mu1 off by 2.4e-5 of |(mu, mu1)| and P1 by 5.9e-7, one pass later 2e-7 and 1.3e-7)
             bool tight = true;
             if (hp_phase) {
                 const double S = 0.25 * (N - zz);
                 tight = gc || o.occ_tol > 0 || tightened ||
-                        std::fabs(err) <= std::max(2e-7 * S, 1e-10 * N);
+                        (std::fabs(err) <= std::max(1e-6 * S, 1e-10 * N) &&
+                         !(S < (wide_ ? 8.0 : 1.0) && beta * std::fabs(step) > 4e-5));
                 if (occ_ok && pass + 1 >= min_pass) {
-                    if (tight || !(S > 0.05)) {
+                    if (tight || !(S > 0.05) || hp_passes == 3) {
                         done = true;
                         break;
                     }
                     tightened = true;
                 }
-                if (++hp_passes >= 4 + (tightened ? 1 : 0)) break;
+                if (++hp_passes >= 4) break;
             } else {
                 // the pass started from relative step residuals below 1e-6, so it left them
                 // at about 1e-9 or at the split-TF32 floor (or, after three extra passes,
@@ -2457,6 +2501,7 @@ cdmpt_status Solver<T>::solve_as(Context& cx, const double* H0, const double* H1
                 if (form == Form::kRefined && st.mu_iterations + ++newton > o.mu_maxit) break;
                 const double slope = 0.25 * beta * (N - zz);
                 const double dmu = slope > 0 ? -err / slope : 0.0;
+                last_step = dmu;
                 mu += dmu;
                 if (fdx_)   // Z_0 = tanh(Y) is not shifted by a multiple of I: rebuild it
                     CDMPT_TRY(init_z0(cx, H0, mu, s2, s2 * std::max(gmax - mu, mu - gmin), acc));
@@ -2472,6 +2517,7 @@ cdmpt_status Solver<T>::solve_as(Context& cx, const double* H0, const double* H1
     }
     st.mu = mu;
     if (mu_out) *mu_out = mu;
+    last_occ_err_ = gc ? 0.0 : trP - nocc;
     cx.mark(2);
     traj_valid_ = true;
     last_beta_ = beta;
@@ -2578,19 +2624,16 @@ cdmpt_status Solver<T>::solve_as(Context& cx, const double* H0, const double* H1
         cx.mark(3);
 
         if (!gc) CDMPT_TRY(compute_q(cx));
+        const bool mu1_of_q = q_exact();
+        double mu1_q[kMaxD] = {};
+        if (mu1_of_q) CDMPT_TRY(mu1_by_q(cx, H1, D, mu1_q));
         CDMPT_CUDA_TRY(cudaMemsetAsync(sc_ + S_TRQ, 0, (S_NSLOTS - S_TRQ) * sizeof(double),
                                        cx.stream));
         if (!gc) CDMPT_TRY(Ew<T>::trace(Qmu_.x, N, ld, 1, sc_ + S_TRQ, cx.stream));
         CDMPT_TRY(Ew<T>::trace(Z1->x, N, ld, D, sc_ + S_TRZ1, cx.stream));
-        const bool mu1_of_q = q_exact();
-        for (int d = 0; d < D && mu1_of_q; ++d)
-            CDMPT_TRY(Ew<T>::dot_h(Qmu_.x, H1 + (size_t)d * blk_, N, ld, ld, sc_ + S_QH + d,
-                                   cx.stream));
         CDMPT_TRY(read_scalars(cx, sc_, S_NSLOTS));
         const double trQ = cx.pinned[S_TRQ];
         st.trace_Q = trQ;
-        double qh[kMaxD];   // the slots are read back again below
-        for (int d = 0; d < kMaxD; ++d) qh[d] = cx.pinned[S_QH + d];
         for (int d = 0; d < D; ++d) {
             const double trP1 = 0.5 * cx.pinned[S_TRZ1 + d];
             if (!std::isfinite(trP1)) return non_finite("the response");
@@ -2598,7 +2641,7 @@ cdmpt_status Solver<T>::solve_as(Context& cx, const double* H0, const double* H1
             // the mean) that makes it traceless; the one handed out is Tr[Q H1] / Tr Q where
             // Q is the more accurate of the two (see q_exact)
             const double mu1 = (!gc && trQ > 0) ? -trP1 / trQ : 0.0;
-            last_mu1_[d] = mu1_of_q && trQ > 0 ? qh[d] / trQ : mu1 + shift[d];
+            last_mu1_[d] = mu1_of_q && trQ > 0 ? mu1_q[d] : mu1 + shift[d];
             if (mu1_out) mu1_out[d] = last_mu1_[d];
             // P1 = Z1/2 + mu1 Q  <=>  Z1 += 2 mu1 Q
             if (!gc)

@@ -260,6 +260,7 @@ private:
     cdmpt_status occupation(Context& cx, int n, double* trP, double* zz);
     cdmpt_status compute_q(Context& cx);
     static cdmpt_status non_finite(const char* what);
+    cdmpt_status mu1_by_q(Context& cx, const double* H1, int D, double* mu1);
     cdmpt_status read_scalars(Context& cx, const double* dev, int count);
     int engine_of(const Context& cx, int override_engine) const;
     // The engine an M x Nc x K product runs on, and whether a symmetric result (sym) is computed
@@ -313,6 +314,7 @@ private:
     bool orders_ready_ = false;
     std::vector<double> last_mu1_;
     std::vector<double> h1_mean_;    // mean diagonal of the last solve's H1_d (FP32 storage)
+    bool wide_ = false;              // a perturbation of the last solve is large against H0
     double* h1_sums_ = nullptr;      // traces and squares of H1_d (device, 32 doubles)
     int no_memory_N_ = 0;            // smallest N whose pair storage did not fit
     bool refined_ = false;           // the trajectory is refined (pairs, FP64-class residuals)
@@ -327,6 +329,7 @@ private:
     // state of the last solve, for the response's Q and the adjoint
     bool traj_valid_ = false, q_valid_ = false;
     double last_beta_ = 0, last_s2_ = 0;
+    double last_occ_err_ = 0;        // Tr P0 - N_occ
     double last_mu_ = 0, last_rho_ = 0;   // mu and max |z0| over the Gershgorin interval
     bool fdx_ = false;                    // Fermi-Dirac-exact start of the current solve
     double gmin_ = 0, gmax_ = 0;          // Gershgorin interval of H0

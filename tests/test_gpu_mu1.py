@@ -41,6 +41,8 @@ def _error(r, ref):
 @pytest.mark.parametrize("precision", ["fp32", "mixed"])
 @pytest.mark.parametrize("kind,N,seed,beta", [("chain", 175, 6, 33.0), ("chain", 240, 4, 26.0),
                                               ("chain", 530, 2, 30.0), ("chain", 700, 10, 40.0),
+                                              ("chain", 130, 11, 52.1), ("chain", 201, 25, 71.7),
+                                              ("chain", 273, 39, 27.6),
                                               ("banded", 600, 8, 15.0), ("banded", 1200, 4, 27.0)])
 def test_mu1_of_wide_perturbations(cuda, cdmpt_lib, kind, N, seed, beta, precision):
     p, ref = _system(kind, N, seed, beta), _reference(kind, N, seed, beta)
