@@ -498,10 +498,10 @@ def run_ours(args):
             "data": "synthetic",
             "config": {"workload": WORKLOAD, "precision": args.precision,
                        "gemm": {"fp32": "tcgen05 3xTF32", "fp64": "CUDA-core DFMA",
-                                "mixed": "tcgen05 TF32 sweeps and CG iterations; 3xTF32 "
-                                         "refinement of early steps, response right-hand sides "
-                                         "and restarts; Ozaki BF16-digit (FP64-class) residuals "
-                                         "of the late steps and of dP0/dmu"}[args.precision],
+                                "mixed": "tcgen05 TF32 sweeps and refinement corrections; "
+                                         "3xTF32 residuals of early steps and response; Ozaki "
+                                         "BF16-digit (FP64-class) residuals and step inverses "
+                                         "of the late steps, and dP0/dmu"}[args.precision],
                        "l2": "no flush: working set (trajectory of 29 N x N matrices as pairs "
                              "with their TF32 splits, about 30 GiB) exceeds the 129 MB L2",
                        "parallelism": f"replicas x{world}"},

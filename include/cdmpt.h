@@ -75,7 +75,7 @@ typedef enum {
                              refinement of the pair-stored (hi + lo FP32) trajectory with
                              split-TF32 residuals on the early steps and FP64-class
                              (Ozaki-sliced BF16) residuals on the late ones (fp64_residual);
-                             split-TF32 response right-hand sides */
+                             split-TF32 response; mu1 from FP64-class products */
     CDMPT_MIXED_BF16 = 3  /* as MIXED_TF32 with BF16 products (FP32 accumulation) for the
                              occupation sweeps */
 } cdmpt_precision;
