@@ -1287,6 +1287,8 @@ cdmpt_status alloc_batch(cdmpt_batch* b, int n) {
     drop_graphs(b);
     for (void* p : b->allocs) cudaFree(p);
     b->allocs.clear();
+    b->n_alloc = 0;   // nothing is there until all of it is
+    b->have_H = false;
     b->map_index.clear();
     b->maps_host.clear();
     b->maps_uploaded = 0;

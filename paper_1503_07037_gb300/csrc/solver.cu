@@ -80,15 +80,31 @@ Solver<T>::~Solver() {
     for (void* p : allocs_) cudaFree(p);
 }
 
+// A failed reservation leaves nothing behind: the sizes would otherwise tell the next solve that
+// its buffers are there.
 template <typename T>
 cdmpt_status Solver<T>::reserve(int N, int D, int n, int ckpt, bool pairs) {
+    const cdmpt_status s = reserve_all(N, D, n, ckpt, pairs);
+    if (s == CDMPT_OK) return s;
+    for (void* p : allocs_) cudaFree(p);
+    allocs_.clear();
+    Z_.clear();
+    W_.clear();
+    N_ = D_ = n_ = rows_cap_ = 0;
+    pairs_ = orders_ready_ = oz64_ready_ = traj_valid_ = q_valid_ = false;
+    return s;
+}
+
+template <typename T>
+cdmpt_status Solver<T>::reserve_all(int N, int D, int n, int ckpt, bool pairs) {
     const int ld_new = (N + 31) / 32 * 32;
     const int rows_needed = std::max(1, D) * N;
     pairs = pairs && sizeof(T) == 4 && ckpt == 0;
     seg_ = -1;
-    // with checkpoints the trajectory views are laid out for exactly n steps
+    // with checkpoints the trajectory views are laid out for exactly n steps; a solve without
+    // refinement runs in the buffers of one with it, so that a program may alternate
     if (N == N_ && D <= D_ && (ckpt == 0 ? n <= n_ : n == n_) && ckpt == ck_ && ld == ld_new &&
-        rows_cap_ >= rows_needed && pairs == pairs_)
+        rows_cap_ >= rows_needed && (pairs_ || !pairs))
         return CDMPT_OK;
     for (void* p : allocs_) cudaFree(p);
     allocs_.clear();
@@ -215,7 +231,11 @@ cdmpt_status Solver<T>::reserve(int N, int D, int n, int ckpt, bool pairs) {
     }
     traj_valid_ = q_valid_ = false;
     void* p = nullptr;
-    if (cudaMalloc(&p, S_NSLOTS * sizeof(double)) != cudaSuccess) return CDMPT_ERR_OOM;
+    if (cudaMalloc(&p, S_NSLOTS * sizeof(double)) != cudaSuccess) {
+        cudaGetLastError();
+        set_error("device allocation of the solver's scalars failed");
+        return CDMPT_ERR_OOM;
+    }
     allocs_.push_back(p);
     sc_ = (double*)p;
     return CDMPT_OK;

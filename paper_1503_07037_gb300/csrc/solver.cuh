@@ -147,6 +147,7 @@ public:
     int ld = 0;
 
 private:
+    cdmpt_status reserve_all(int N, int D, int n, int ckpt, bool pairs);
     // How a solve runs: as its options say; an FP32 solve with the refinement of the mixed
     // precision; or by CG throughout (see solve() in solver.cu).
     enum class Form { kPlain, kRefined, kCg };
