@@ -3,6 +3,7 @@
 The memory is taken by an allocation of the test's own; N = 1024, n = 14, FP32: 0.46 GB without the
 low parts and digits of a refined trajectory (0.1 GB more), 60 MB for H0 and H1 and their copies.
 """
+import contextlib
 import math
 
 import numpy as np
@@ -17,17 +18,21 @@ ERR_OOM = 7
 MB = 1 << 20
 
 
+@contextlib.contextmanager
 def _leave(free_bytes):
-    """Allocations that leave about free_bytes of the device."""
+    """Allocations that leave about free_bytes of the device, given back at the end."""
     import torch
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     held = []
-    while True:
-        rest = torch.cuda.mem_get_info()[0] - free_bytes
-        if rest < 4 * MB:
-            return held
-        held.append(torch.empty(min(rest, 64 << 30), dtype=torch.uint8, device="cuda"))
+    try:
+        while torch.cuda.mem_get_info()[0] - free_bytes >= 4 * MB:
+            rest = torch.cuda.mem_get_info()[0] - free_bytes
+            held.append(torch.empty(min(rest, 64 << 30), dtype=torch.uint8, device="cuda"))
+        yield
+    finally:
+        held.clear()
+        torch.cuda.empty_cache()
 
 
 @pytest.fixture
@@ -48,14 +53,11 @@ def test_solve_after_out_of_memory(cuda, cdmpt_lib, chain, precision):
     p, ref = chain
     with cdmpt_lib.Handle(precision=precision) as h:
         h.set_H(p.H0, p.H1)
-        held = _leave(150 * MB)
-        for _ in range(3):      # a second call must not take the first one's buffers for granted
-            with pytest.raises(cdmpt_lib.CdmptError) as e:
-                h.solve(p.beta, p.nocc, p.n, want_P0=False, want_P1=False)
-            assert e.value.status == ERR_OOM
-        del held
-        import torch
-        torch.cuda.empty_cache()
+        with _leave(150 * MB):
+            for _ in range(3):      # a second call must not take the first one's buffers as there
+                with pytest.raises(cdmpt_lib.CdmptError) as e:
+                    h.solve(p.beta, p.nocc, p.n, want_P0=False, want_P1=False)
+                assert e.value.status == ERR_OOM
         _check(h.solve(p.beta, p.nocc, p.n), p, ref, 1e-5)
 
 
@@ -76,12 +78,11 @@ def test_fp32_without_room_for_the_refinement(cuda, cdmpt_lib, chain):
             mixed.solve(p.beta, p.nocc, p.n)
             refined = free0 - torch.cuda.mem_get_info()[0]
         assert refined > need
-        held = _leave((need + refined) // 2)
-        for _ in range(2):
-            r = h.solve(p.beta, p.nocc, p.n)
-            assert h.stats()["refine_passes"] == 0
-            _check(r, p, ref, 1e-5)
-        del held
+        with _leave((need + refined) // 2):
+            for _ in range(2):
+                r = h.solve(p.beta, p.nocc, p.n)
+                assert h.stats()["refine_passes"] == 0
+                _check(r, p, ref, 1e-5)
 
 
 def test_alternating_perturbations_keep_the_buffers(cuda, cdmpt_lib):
